@@ -9,19 +9,34 @@
 // C_k = min over the matching cameras of (1 - ZNCC) / 2 (lowest camera index
 // on a tie), exactly the sweep's cost but on real-valued images.
 //
-// Kernels (one CTA per 16 x 16 output tile, one thread per output pixel):
-//   soft_fwd_kernel  per pair of planes and camera, warp the tile + window
-//                    halo into shared memory; two-pass window ZNCC per pixel
-//                    (both planes on packed FP32 pairs); minimum over
-//                    cameras; online softmax over planes.
-//   soft_bwd_kernel  recomputes the same costs (bit-identical) while keeping
-//                    each warped sample's bilinear cell and pose derivative,
-//                    forms dL/dC_k, spreads dL/dZNCC over both windows as
-//                    separable box sums of per-pixel coefficients, then per
-//                    warped halo sample scatters dL/dI to the 4 bilinear
-//                    texels and adds dL/dw times the sample's pose
+// Kernels (planes in pairs on packed FP32):
+//   soft_fwd_kernel  32 x 16 output pixels: per pair of planes and camera,
+//                    warp the tile + window halo into shared memory; two-pass
+//                    window ZNCC, two pixels per thread so that they share the
+//                    window rows they load; minimum over cameras; online
+//                    softmax over planes.
+//   soft_bwd_kernel  16 x 16 output pixels: recomputes the same costs (bit-
+//                    identical), forms dL/dC_k, spreads dL/dZNCC over both
+//                    windows as separable box sums of per-pixel coefficients,
+//                    then per warped halo sample with a gradient warps it
+//                    again with its derivative, scatters dL/dI to the 4
+//                    bilinear texels and adds dL/dw times the sample's pose
 //                    derivative to a left perturbation (w, v) of each
 //                    ref_to_cam pose (CTA reduction, FP64 atomics).
+// Both are bound by instruction issue and latency (DRAM holds the images and
+// ray table once).  A forward and backward pass through autograd, 640 x 512,
+// 128 planes, 2 cameras: 5964 -> 4233 us; 96 x 80, 32 planes: 689 -> 597 us.
+// Before: one pixel per thread, general divisions and square roots (their
+// slow-path branches serialise a thread's samples), the reference window's
+// sums repeated per plane, and a backward of one plane at a time with seven
+// barriers and its chain data in shared memory.
+//
+// Low-texture windows have coefficients so large that a changed rounding of a
+// cost or a coefficient shows in the image gradients (2e-5 .. 7e-5 of their
+// norm in a build that merged coefficient fields and softmax parts), so costs,
+// softmax, box sums and the pose accumulators keep one order whatever the
+// tiling.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -33,13 +48,12 @@ int build_rays(const ps_camera& cam, float4* rays, double* max_angle);
 
 namespace {
 
-constexpr int DT = 16;                 // output tile edge
-constexpr int DNT = DT * DT;           // threads per CTA
-
 struct DiffCam {
-    float R[9], t[3];
-    CamF c;
+    int width, height;
     const float* img;
+    float r2_max;
+    // projection constants, and those of its derivative, as (value, value) pairs
+    float2 R2[9], t2[3], xi, fx, fy, cx, cy, k1, k2, k2x2, p1, p1x2, p1x6, p2, p2x2, p2x6, lim;
 };
 
 struct DiffP {
@@ -51,54 +65,38 @@ struct DiffP {
     DiffCam cams[PS_MAX_CAMS];
 };
 
-// Projection of X_j (camera frame) with the unified model and distortion;
-// false where the point does not project (the sweep's validity rules).
-__device__ __forceinline__ bool project_f(const CamF& c, float X, float Y, float Z, float* u, float* v,
-                                          float* n_out) {
-    float n = sqrtf(fmaf(X, X, fmaf(Y, Y, Z * Z)));
-    float inv = 1.0f / fmaf(c.xi, n, Z);
-    float mx = X * inv, my = Y * inv;
-    float r2 = fmaf(mx, mx, my * my);
-    float rad = fmaf(r2, fmaf(c.k2, r2, c.k1), 1.0f);
-    float mxy = mx * my;
-    float xd = fmaf(mx, rad, fmaf(2.0f * c.p1, mxy, c.p2 * fmaf(2.0f * mx, mx, r2)));
-    float yd = fmaf(my, rad, fmaf(c.p1, fmaf(2.0f * my, my, r2), 2.0f * c.p2 * mxy));
-    *u = fmaf(c.fx, xd, c.cx);
-    *v = fmaf(c.fy, yd, c.cy);
-    *n_out = n;
-    return (Z > c.lim * n) && (r2 <= c.r2_max);
+// Correctly rounded reciprocals, quotients and square roots without the
+// branches of the general forms (which serialise the samples of a thread),
+// for pairs: from an approximation y0 of 1 / b, y = RN(y0 + y0 (1 - b y0)); a
+// quotient is q + (a - b q) y with q = RN(a y), a square root g + (a - g g) h
+// with g = RN(a y), h = y / 2, y an approximation of 1 / sqrt(a) (P. Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000
+// processor", 1990).  Compared with __frcp_rn, __fsqrt_rn and __fdiv_rn: no
+// difference over every mantissa at 8 exponents, every mantissa at 71, and
+// 10^9 random quotients.  Operands are normal numbers; a zero or infinite
+// operand gives NaN, which every caller rejects like the infinity.
+__device__ __forceinline__ float2 rcp_rn2(float2 b) {
+    const float2 y = make_float2(rcp_ftz(b.x), rcp_ftz(b.y));
+    return fma2(y, fma2(neg2(b), y, dup2(1.0f)), y);
 }
-
-// g = J^T (gu, gv) for the projection Jacobian J = d(u, v)/dX at X (camera
-// frame), by reverse-mode differentiation of project_f instead of forming J:
-// the adjoints of the distorted point, of the normalised point (mx, my),
-// then of X through mx = X / den, my = Y / den, den = xi |X| + Z.
-__device__ __forceinline__ void project_vjp_f(const CamF& c, float X, float Y, float Z, float gu, float gv,
-                                              float g[3]) {
-    const float n = sqrtf(fmaf(X, X, fmaf(Y, Y, Z * Z)));
-    const float id = 1.0f / fmaf(c.xi, n, Z);
-    const float mx = X * id, my = Y * id;
-    const float r2 = fmaf(mx, mx, my * my);
-    const float rad = fmaf(r2, fmaf(c.k2, r2, c.k1), 1.0f), drad = fmaf(2.0f * c.k2, r2, c.k1);
-    // d(xd, yd)/d(mx, my) = [[a, b], [b, d]]
-    const float a = rad + 2.0f * mx * mx * drad + 2.0f * c.p1 * my + 6.0f * c.p2 * mx;
-    const float b = 2.0f * mx * my * drad + 2.0f * c.p1 * mx + 2.0f * c.p2 * my;
-    const float d = rad + 2.0f * my * my * drad + 6.0f * c.p1 * my + 2.0f * c.p2 * mx;
-    const float gxd = gu * c.fx, gyd = gv * c.fy;
-    const float gmx = fmaf(gxd, a, gyd * b), gmy = fmaf(gxd, b, gyd * d);
-    const float sden = fmaf(gmx, mx, gmy * my) * id;  // -dL/dden
-    const float xn = c.xi / n;                        // d(xi n)/dX = xi X / n
-    g[0] = fmaf(gmx, id, -sden * xn * X);
-    g[1] = fmaf(gmy, id, -sden * xn * Y);
-    g[2] = -sden * fmaf(xn, Z, 1.0f);
+// a / b for y = rcp_rn2(b)
+__device__ __forceinline__ float2 div_rn2(float2 a, float2 b, float2 y) {
+    const float2 q = mul2(a, y);
+    return fma2(fma2(neg2(b), q, a), y, q);
 }
-
-// The warp of halo position (gx, gy) through plane P into camera C: the
-// point in the camera frame, the pixel and the bilinear sample (NaN when
-// invalid: no ray, plane behind the ray, no projection, outside the image).
-struct Warp {
-    float X, Y, Z, u, v, w;
-};
+__device__ __forceinline__ float2 sqrt_rn2(float2 a) {
+    const float2 y = make_float2(rsqrt_ftz(a.x), rsqrt_ftz(a.y));
+    const float2 g = mul2(a, y);
+    return fma2(fma2(neg2(g), g, a), mul2(y, dup2(0.5f)), g);
+}
+__device__ __forceinline__ float rcp_rn(float b) {
+    const float y = rcp_ftz(b);
+    return __fmaf_rn(y, __fmaf_rn(-b, y, 1.0f), y);
+}
+__device__ __forceinline__ float div_rn(float a, float b, float y) {
+    const float q = __fmul_rn(a, y);
+    return __fmaf_rn(__fmaf_rn(-b, q, a), y, q);
+}
 
 // n . r of a plane and a ray.  The plane's offset along the ray, and the
 // bilinear blend below, are written with explicit roundings so that every
@@ -115,229 +113,291 @@ __device__ __forceinline__ float bilerp(float ax, float ay, float i00, float i10
     return __fmaf_rn(ay, bot, __fmul_rn(by, top));
 }
 
-// Bilinear sample of camera C at (u, v), NaN outside [0, W-1] x [0, H-1].
-__device__ __forceinline__ float sample_uv(const DiffCam& C, float u, float v) {
-    if (!(u >= 0.0f && u <= (float)(C.c.width - 1) && v >= 0.0f && v <= (float)(C.c.height - 1)))
-        return __int_as_float(0x7fc00000);
-    int x0 = (int)floorf(u), y0 = (int)floorf(v);
-    int x1 = min(x0 + 1, C.c.width - 1), y1 = min(y0 + 1, C.c.height - 1);
-    float ax = u - (float)x0, ay = v - (float)y0;
-    const float* I = C.img;
-    return bilerp(ax, ay, I[(size_t)y0 * C.c.width + x0], I[(size_t)y0 * C.c.width + x1],
-                  I[(size_t)y1 * C.c.width + x0], I[(size_t)y1 * C.c.width + x1]);
-}
-
-__device__ __forceinline__ Warp warp_at(const DiffP& P, const DiffCam& C, const PlaneD& pl, int gx, int gy) {
-    const float nan = __int_as_float(0x7fc00000);
-    Warp o{0.f, 0.f, 0.f, 0.f, 0.f, nan};
-    if (gx < 0 || gy < 0 || gx >= P.W || gy >= P.H) return o;
-    float4 r = P.rays[(size_t)gy * P.W + gx];
-    float nr = plane_dot(pl, r);
-    if (!(nr > 0.0f)) return o;
-    float lam = pl.d / nr;
-    float x = lam * r.x, y = lam * r.y, z = lam * r.z;
-    o.X = fmaf(C.R[0], x, fmaf(C.R[1], y, fmaf(C.R[2], z, C.t[0])));
-    o.Y = fmaf(C.R[3], x, fmaf(C.R[4], y, fmaf(C.R[5], z, C.t[1])));
-    o.Z = fmaf(C.R[6], x, fmaf(C.R[7], y, fmaf(C.R[8], z, C.t[2])));
-    float n;
-    if (!project_f(C.c, o.X, o.Y, o.Z, &o.u, &o.v, &n)) return o;
-    o.w = sample_uv(C, o.u, o.v);
+// Halo position r (its ray) through the planes p0 (lane x) and p1 (lane y)
+// into camera C: the point in the camera frame, the projection (unified
+// model, then distortion) with its intermediate values, and whether each
+// lane projects (plane before the ray, sphere side, distortion range).
+struct Proj {
+    float2 X, Y, Z, n, inv, mx, my, r2, rad, u, v;
+    bool ok0, ok1;
+};
+__device__ __forceinline__ Proj project_pair(const DiffCam& C, const PlaneD& p0, const PlaneD& p1, const float4& r) {
+    Proj o;
+    const float2 nr = make_float2(plane_dot(p0, r), plane_dot(p1, r));
+    const float2 lam = div_rn2(make_float2(p0.d, p1.d), nr, rcp_rn2(nr));
+    const float2 x = mul2(lam, dup2(r.x)), y = mul2(lam, dup2(r.y)), z = mul2(lam, dup2(r.z));
+    o.X = fma2(C.R2[0], x, fma2(C.R2[1], y, fma2(C.R2[2], z, C.t2[0])));
+    o.Y = fma2(C.R2[3], x, fma2(C.R2[4], y, fma2(C.R2[5], z, C.t2[1])));
+    o.Z = fma2(C.R2[6], x, fma2(C.R2[7], y, fma2(C.R2[8], z, C.t2[2])));
+    o.n = sqrt_rn2(fma2(o.X, o.X, fma2(o.Y, o.Y, mul2(o.Z, o.Z))));
+    o.inv = rcp_rn2(fma2(C.xi, o.n, o.Z));
+    o.mx = mul2(o.X, o.inv);
+    o.my = mul2(o.Y, o.inv);
+    o.r2 = fma2(o.mx, o.mx, mul2(o.my, o.my));
+    o.rad = fma2(o.r2, fma2(C.k2, o.r2, C.k1), dup2(1.0f));
+    const float2 mxy = mul2(o.mx, o.my);
+    const float2 xd = fma2(o.mx, o.rad, fma2(C.p1x2, mxy, mul2(C.p2, fma2(add2(o.mx, o.mx), o.mx, o.r2))));
+    const float2 yd = fma2(o.my, o.rad, fma2(C.p1, fma2(add2(o.my, o.my), o.my, o.r2), mul2(C.p2x2, mxy)));
+    o.u = fma2(C.fx, xd, C.cx);
+    o.v = fma2(C.fy, yd, C.cy);
+    const float2 ln = mul2(C.lim, o.n);
+    o.ok0 = nr.x > 0.0f && o.Z.x > ln.x && o.r2.x <= C.r2_max;
+    o.ok1 = nr.y > 0.0f && o.Z.y > ln.y && o.r2.y <= C.r2_max;
     return o;
 }
 
-// warp_at for two planes at once (lane x: p0, lane y: p1): the samples only,
-// with the transform and the projection on packed FP32 pairs.  Per lane
-// every operation and rounding is that of warp_at (2 m = m + m exactly), so
-// each sample is bit-identical to warp_at's.
-__device__ __forceinline__ float2 warp_pair(const DiffP& P, const DiffCam& C, const PlaneD& p0, const PlaneD& p1,
-                                            int gx, int gy) {
-    const float nan = __int_as_float(0x7fc00000);
-    if (gx < 0 || gy < 0 || gx >= P.W || gy >= P.H) return make_float2(nan, nan);
-    const float4 r = P.rays[(size_t)gy * P.W + gx];
-    const float nr0 = plane_dot(p0, r), nr1 = plane_dot(p1, r);
-    const bool f0 = nr0 > 0.0f, f1 = nr1 > 0.0f;
-    if (!(f0 || f1)) return make_float2(nan, nan);
-    const float2 lam = make_float2(p0.d / nr0, p1.d / nr1);
-    const float2 x = mul2(lam, dup2(r.x)), y = mul2(lam, dup2(r.y)), z = mul2(lam, dup2(r.z));
-    const float2 X = fma2(dup2(C.R[0]), x, fma2(dup2(C.R[1]), y, fma2(dup2(C.R[2]), z, dup2(C.t[0]))));
-    const float2 Y = fma2(dup2(C.R[3]), x, fma2(dup2(C.R[4]), y, fma2(dup2(C.R[5]), z, dup2(C.t[1]))));
-    const float2 Z = fma2(dup2(C.R[6]), x, fma2(dup2(C.R[7]), y, fma2(dup2(C.R[8]), z, dup2(C.t[2]))));
-    const CamF& c = C.c;
-    const float2 n2 = fma2(X, X, fma2(Y, Y, mul2(Z, Z)));
-    const float2 n = make_float2(sqrtf(n2.x), sqrtf(n2.y));
-    const float2 den = fma2(dup2(c.xi), n, Z);
-    const float2 inv = make_float2(1.0f / den.x, 1.0f / den.y);
-    const float2 mx = mul2(X, inv), my = mul2(Y, inv);
-    const float2 r2 = fma2(mx, mx, mul2(my, my));
-    const float2 rad = fma2(r2, fma2(dup2(c.k2), r2, dup2(c.k1)), dup2(1.0f));
-    const float2 mxy = mul2(mx, my);
-    const float2 xd = fma2(mx, rad, fma2(dup2(2.0f * c.p1), mxy, mul2(dup2(c.p2), fma2(add2(mx, mx), mx, r2))));
-    const float2 yd = fma2(my, rad, fma2(dup2(c.p1), fma2(add2(my, my), my, r2), mul2(dup2(2.0f * c.p2), mxy)));
-    const float2 u = fma2(dup2(c.fx), xd, dup2(c.cx)), v = fma2(dup2(c.fy), yd, dup2(c.cy));
-    const float2 ln = mul2(dup2(c.lim), n);
-    const bool g0 = f0 && (Z.x > ln.x) && (r2.x <= c.r2_max), g1 = f1 && (Z.y > ln.y) && (r2.y <= c.r2_max);
-    return make_float2(g0 ? sample_uv(C, u.x, v.x) : nan, g1 ? sample_uv(C, u.y, v.y) : nan);
+// The bilinear cell of camera C at (u, v), clamped into the image: corner
+// offsets and weights; false when (u, v) lies outside [0, W-1] x [0, H-1].
+struct Cell {
+    int i00, i10, i01, i11;
+    float ax, ay;
+};
+__device__ __forceinline__ bool cell_at(const DiffCam& C, float u, float v, Cell& c) {
+    const float uc = fminf(fmaxf(u, 0.0f), (float)(C.width - 1)), vc = fminf(fmaxf(v, 0.0f), (float)(C.height - 1));
+    int x = (int)uc, y = (int)vc;
+    if (!PS_DCHECK(x >= 0 && y >= 0 && x < C.width && y < C.height, CHK_GATHER)) x = y = 0;
+    const int dx = x < C.width - 1 ? 1 : 0, dy = y < C.height - 1 ? C.width : 0;
+    c.i00 = y * C.width + x;
+    c.i10 = c.i00 + dx;
+    c.i01 = c.i00 + dy;
+    c.i11 = c.i01 + dx;
+    c.ax = uc - (float)x;
+    c.ay = vc - (float)y;
+    return uc == u && vc == v;
 }
 
-// Two-pass ZNCC of the pixel's window: reference samples R and warped
-// samples Wv in the halo layout (row stride DS).  False when a sample is
-// invalid or a window is flat.
-struct Zn {
-    float z, ma, mb, va, vb, sab;
+// Samples of camera C at a halo position through two planes (lane x: p0, lane
+// y: p1); NaN where invalid (no ray, plane behind the ray, no projection,
+// outside the image).  The gathers are clamped into the image and always
+// issued, so nothing branches and a thread's positions overlap.
+__device__ __forceinline__ float2 warp_pair(const DiffCam& C, const PlaneD& p0, const PlaneD& p1, const float4& r) {
+    const float nan = __int_as_float(0x7fc00000);
+    const Proj o = project_pair(C, p0, p1, r);
+    Cell a, b;
+    const bool in0 = cell_at(C, o.u.x, o.v.x, a), in1 = cell_at(C, o.u.y, o.v.y, b);
+    const float* I = C.img;
+    const float w0 = bilerp(a.ax, a.ay, I[a.i00], I[a.i10], I[a.i01], I[a.i11]);
+    const float w1 = bilerp(b.ax, b.ay, I[b.i00], I[b.i10], I[b.i01], I[b.i11]);
+    return make_float2(o.ok0 && in0 ? w0 : nan, o.ok1 && in1 ? w1 : nan);
+}
+
+// ----------------------------------------------------------------- tiles
+//
+// A CTA of ST threads works on SW columns of output pixels: thread t owns the
+// PX pixels of column t % SW from row PX (t / SW), so that a window row that
+// several of them hold is loaded once.  Planes go in pairs (lane x: the first
+// plane, lane y: the second) on packed FP32.
+constexpr int ST = 256;  // threads per CTA
+
+template <int RHO_, int SW_, int PX_>
+struct Tile {
+    static constexpr int RHO = RHO_, SW = SW_, PX = PX_;
+    static constexpr int TH = ST / SW * PX;                // output rows
+    static constexpr int HWC = SW + 2 * RHO, HH = TH + 2 * RHO, NPOS = HWC * HH;
+    static constexpr int RPT = (NPOS + ST - 1) / ST;       // halo positions per thread
+    static constexpr int N = (2 * RHO + 1) * (2 * RHO + 1);
 };
 
-// Shared-memory row stride of the halo buffers: 48 = 16 (mod 32), so the two
-// output rows of a warp (16 pixels each) read disjoint banks.
-constexpr int DS = 48;
-
-template <int RHO>
-__device__ __forceinline__ bool window_zncc(const float* R, const float* Wv, int lx, int ly, Zn* o) {
-    constexpr int N = (2 * RHO + 1) * (2 * RHO + 1);
-    float sa = 0.f, sb = 0.f;
-    bool ok = true;
+// Mean and sum of squared deviations of the reference windows of a thread's
+// PX pixels (R: halo layout, the first pixel's window at lx, ly).  One pass
+// each in row-major window order.
+template <class G>
+__device__ __forceinline__ void ref_windows(const float* R, int lx, int ly, float (&ma)[G::PX], float (&va)[G::PX]) {
+    constexpr int RHO = G::RHO, PX = G::PX;
 #pragma unroll
-    for (int dy = 0; dy <= 2 * RHO; ++dy)
+    for (int i = 0; i < PX; ++i) {
+        float s = 0.f;
+        for (int dy = 0; dy <= 2 * RHO; ++dy)
 #pragma unroll
-        for (int dx = 0; dx <= 2 * RHO; ++dx) {
-            const int q = (ly + dy) * DS + lx + dx;
-            float b = Wv[q];
-            ok &= !isnan(b);
-            sa += R[q];
-            sb += b;
-        }
-    if (!ok) return false;
-    float ma = sa / (float)N, mb = sb / (float)N;
-    float cov = 0.f, va = 0.f, vb = 0.f;
+            for (int dx = 0; dx <= 2 * RHO; ++dx) s += R[(ly + i + dy) * G::HWC + lx + dx];
+        const float m = s / (float)G::N;
+        float v = 0.f;
+        for (int dy = 0; dy <= 2 * RHO; ++dy)
 #pragma unroll
-    for (int dy = 0; dy <= 2 * RHO; ++dy)
-#pragma unroll
-        for (int dx = 0; dx <= 2 * RHO; ++dx) {
-            const int q = (ly + dy) * DS + lx + dx;
-            float ea = R[q] - ma, eb = Wv[q] - mb;
-            cov = fmaf(ea, eb, cov);
-            va = fmaf(ea, ea, va);
-            vb = fmaf(eb, eb, vb);
-        }
-    if (va < (float)N * 1e-8f || vb < (float)N * 1e-8f) return false;
-    o->sab = sqrtf(va * vb);
-    o->z = cov / o->sab;
-    o->ma = ma;
-    o->mb = mb;
-    o->va = va;
-    o->vb = vb;
-    return true;
-}
-
-// window_zncc for two planes at once: warped pairs Wv (lane x: the first
-// plane, lane y: the second), one reference window.  The reference sums are
-// shared; per lane every sum and rounding is window_zncc's, so z is
-// bit-identical to it.  ok0 / ok1: the lanes' validity.
-template <int RHO>
-__device__ __forceinline__ float2 window_zncc2(const float* R, const float2* Wv, int lx, int ly, bool* ok0, bool* ok1) {
-    constexpr int N = (2 * RHO + 1) * (2 * RHO + 1);
-    float sa = 0.f;
-    float2 sb = dup2(0.f);
-    bool v0 = true, v1 = true;
-#pragma unroll
-    for (int dy = 0; dy <= 2 * RHO; ++dy)
-#pragma unroll
-        for (int dx = 0; dx <= 2 * RHO; ++dx) {
-            const int q = (ly + dy) * DS + lx + dx;
-            const float2 b = Wv[q];
-            v0 &= !isnan(b.x);
-            v1 &= !isnan(b.y);
-            sa += R[q];
-            sb = add2(sb, b);
-        }
-    *ok0 = *ok1 = false;
-    if (!(v0 || v1)) return dup2(0.f);
-    const float ma = sa / (float)N;
-    const float2 nmb = make_float2(-(sb.x / (float)N), -(sb.y / (float)N));
-    float va = 0.f;
-    float2 cov = dup2(0.f), vb = dup2(0.f);
-#pragma unroll
-    for (int dy = 0; dy <= 2 * RHO; ++dy)
-#pragma unroll
-        for (int dx = 0; dx <= 2 * RHO; ++dx) {
-            const int q = (ly + dy) * DS + lx + dx;
-            const float ea = R[q] - ma;
-            const float2 eb = add2(Wv[q], nmb);
-            cov = fma2(dup2(ea), eb, cov);
-            va = fmaf(ea, ea, va);
-            vb = fma2(eb, eb, vb);
-        }
-    const float lim = (float)N * 1e-8f;
-    *ok0 = v0 && !(va < lim || vb.x < lim);
-    *ok1 = v1 && !(va < lim || vb.y < lim);
-    return make_float2(cov.x / sqrtf(va * vb.x), cov.y / sqrtf(va * vb.y));
-}
-
-// Window 5: three CTAs per SM (80 registers, a small spill) measured faster
-// than two without the limit.
-template <int RHO>
-__global__ void __launch_bounds__(DNT, RHO == 2 ? 3 : 1) soft_fwd_kernel(const __grid_constant__ DiffP P, float* range, float* cost,
-                                                      float* aux) {
-    constexpr int HW = DT + 2 * RHO, NPOS = HW * HW;
-    __shared__ float Rs[HW * DS];
-    __shared__ float2 W2[HW * DS];  // warped samples of a pair of planes
-    const int tid = threadIdx.x, lx = tid % DT, ly = tid / DT;
-    const int x0 = blockIdx.x * DT - RHO, y0 = blockIdx.y * DT - RHO;
-    const int gx = blockIdx.x * DT + lx, gy = blockIdx.y * DT + ly;
-    for (int p = tid; p < NPOS; p += DNT) {
-        const int hx = p % HW, hy = p / HW, x = x0 + hx, y = y0 + hy;
-        Rs[hy * DS + hx] = (x >= 0 && y >= 0 && x < P.W && y < P.H) ? P.ref[(size_t)y * P.W + x] : 0.0f;
+            for (int dx = 0; dx <= 2 * RHO; ++dx) {
+                const float e = R[(ly + i + dy) * G::HWC + lx + dx] - m;
+                v = fmaf(e, e, v);
+            }
+        ma[i] = m;
+        va[i] = v;
     }
-    const bool in = gx < P.W && gy < P.H;
-    float4 ray = in ? P.rays[(size_t)gy * P.W + gx] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const bool use = in && gx >= RHO && gy >= RHO && gx < P.W - RHO && gy < P.H - RHO && !isnan(ray.x);
+}
+
+// Two-pass ZNCC sums of both planes for a thread's PX pixels under each
+// other: warped pairs W, reference R (halo layout).  Per pixel and plane the
+// sums run over the window in row-major order; a window row shared by
+// several pixels is loaded once.  An invalid sample is NaN and makes the
+// mean NaN.
+template <class G>
+__device__ __forceinline__ void pair_windows(const float* R, const float2* W, int lx, int ly, const float (&ma)[G::PX],
+                                             float2 (&mb)[G::PX], float2 (&cov)[G::PX], float2 (&vb)[G::PX]) {
+    constexpr int RHO = G::RHO, PX = G::PX;
+#pragma unroll
+    for (int i = 0; i < PX; ++i) mb[i] = cov[i] = vb[i] = dup2(0.f);
+#pragma unroll
+    for (int y = 0; y < 2 * RHO + PX; ++y)
+#pragma unroll
+        for (int dx = 0; dx <= 2 * RHO; ++dx) {
+            const float2 b = W[(ly + y) * G::HWC + lx + dx];
+#pragma unroll
+            for (int i = 0; i < PX; ++i)
+                if (y - i >= 0 && y - i <= 2 * RHO) mb[i] = add2(mb[i], b);
+        }
+    float2 nmb[PX];
+#pragma unroll
+    for (int i = 0; i < PX; ++i) {
+        mb[i] = div_rn2(mb[i], dup2((float)G::N), dup2(1.0f / (float)G::N));
+        nmb[i] = neg2(mb[i]);
+    }
+    asm volatile("" ::: "memory");  // the second pass loads again: keeping the window in registers would spill
+#pragma unroll
+    for (int y = 0; y < 2 * RHO + PX; ++y)
+#pragma unroll
+        for (int dx = 0; dx <= 2 * RHO; ++dx) {
+            const float2 b = W[(ly + y) * G::HWC + lx + dx];
+            const float a = R[(ly + y) * G::HWC + lx + dx];
+#pragma unroll
+            for (int i = 0; i < PX; ++i)
+                if (y - i >= 0 && y - i <= 2 * RHO) {
+                    const float2 ea = dup2(a - ma[i]), eb = add2(b, nmb[i]);
+                    cov[i] = fma2(ea, eb, cov[i]);
+                    vb[i] = fma2(eb, eb, vb[i]);
+                }
+        }
+}
+
+// The tile's reference samples (zero outside the image).
+template <class G>
+__device__ __forceinline__ void load_ref(const DiffP& P, int x0, int y0, float* R) {
+    for (int p = threadIdx.x; p < G::NPOS; p += blockDim.x) {
+        const int hy = p / G::HWC, hx = p - hy * G::HWC, x = x0 + hx, y = y0 + hy;
+        R[p] = (x >= 0 && y >= 0 && x < P.W && y < P.H) ? P.ref[(size_t)y * P.W + x] : 0.0f;
+    }
+}
+
+// Ray of image position (x, y), NaN outside the image.
+__device__ __forceinline__ float4 ray_at(const DiffP& P, int x, int y) {
+    const float nan = __int_as_float(0x7fc00000);
+    return x >= 0 && y >= 0 && x < P.W && y < P.H ? P.rays[(size_t)y * P.W + x] : make_float4(nan, nan, nan, 0.f);
+}
+
+// Warped sample pairs of the halo, every camera, by the ST threads tid.
+template <class G>
+__device__ __forceinline__ void warp_tile(const DiffP& P, const PlaneD& pl0, const PlaneD& pl1, int x0, int y0, int tid,
+                                          float2* W2) {
+    for (int j = 0; j < P.n_cams; ++j)
+#pragma unroll
+        for (int i = 0; i < G::RPT; ++i) {
+            const int p = tid + i * ST;
+            if (p < G::NPOS) W2[j * G::NPOS + p] = warp_pair(P.cams[j], pl0, pl1, ray_at(P, x0 + p % G::HWC, y0 + p / G::HWC));
+        }
+}
+
+// The forward's CTA: FG groups of ST threads share a tile and take alternate
+// pairs of planes; each pixel's costs of a round of ROUND planes wait in
+// shared memory, then every thread goes over them in plane order for the
+// pixels it owns there.  The online softmax thus adds the planes one by one
+// in plane order, while two groups halve the time of a tile: 640 tiles of 32
+// x 16 pixels (640 x 512) are 4.2 waves of one 512-thread CTA per SM instead
+// of 2.1 waves of two of 256 threads.
+constexpr int FG = 2;
+constexpr int ROUND = 16;
+
+template <class G>
+__global__ void __launch_bounds__(FG * ST, 1) soft_fwd_kernel(const __grid_constant__ DiffP P, float* range, float* cost,
+                                                              float* aux) {
+    constexpr int RHO = G::RHO, PX = G::PX, SW = G::SW, NPIX = ST * PX;
+    constexpr int OWN = (NPIX + FG * ST - 1) / (FG * ST);             // pixels a thread owns in the softmax
+    extern __shared__ __align__(16) float sm[];
+    float* Cs = sm;                                                   // [ROUND][NPIX] costs (inf = invalid)
+    const int group = threadIdx.x / ST, tid = threadIdx.x % ST;
+    float2* W2 = reinterpret_cast<float2*>(Cs + ROUND * NPIX) + group * P.n_cams * G::NPOS;  // [n_cams][NPOS] warped pairs
+    float* R = Cs + ROUND * NPIX + 2 * FG * P.n_cams * G::NPOS;       // [NPOS] reference
+    const int lx = tid % SW, ly = tid / SW * PX;
+    const int bx = blockIdx.x * SW, by = blockIdx.y * G::TH;
+    load_ref<G>(P, bx - RHO, by - RHO, R);
+    __syncthreads();
+    float ma[PX], va[PX];
+    ref_windows<G>(R, lx, ly, ma, va);
     const float inf = __int_as_float(0x7f800000);
-    float cmin = inf, Z = 0.f, Nr = 0.f;
-    // planes in pairs (k, k + 1), warped and matched together on packed FP32
-    for (int k = 0; k < P.K; k += 2) {
-        const int np = min(2, P.K - k);
-        const PlaneD pl0 = P.planes[k], pl1 = P.planes[k + np - 1];
-        float best[2] = {inf, inf};
-        for (int j = 0; j < P.n_cams; ++j) {
-            __syncthreads();
-            for (int p = tid; p < NPOS; p += DNT) {
-                const int hx = p % HW, hy = p / HW;
-                W2[hy * DS + hx] = warp_pair(P, P.cams[j], pl0, pl1, x0 + hx, y0 + hy);
-            }
-            __syncthreads();
-            if (use) {
-                bool ok0, ok1;
-                const float2 z = window_zncc2<RHO>(Rs, W2, lx, ly, &ok0, &ok1);
-                const float c0 = 0.5f * (1.0f - z.x), c1 = 0.5f * (1.0f - z.y);
-                if (ok0 && c0 < best[0]) best[0] = c0;
-                if (ok1 && c1 < best[1]) best[1] = c1;
-            }
-        }
+    const float lim = (float)G::N * 1e-8f, inv_T = __frcp_rn(P.T);
+    float cmin[OWN], Z[OWN], Nr[OWN];
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            if (q >= np || !(best[q] < inf)) continue;
-            const PlaneD& pl = q == 0 ? pl0 : pl1;
-            const float bq = best[q];
-            float rho_k = plane_dot(pl, ray) / pl.d;
-            if (bq < cmin) {  // rescale the running sums to the new minimum
-                float f = cmin < inf ? __expf(-(cmin - bq) / P.T) : 0.f;
-                Z *= f;
-                Nr *= f;
-                cmin = bq;
-            }
-            float e = __expf(-(bq - cmin) / P.T);
-            Z += e;
-            Nr = fmaf(e, rho_k, Nr);
-        }
+    for (int i = 0; i < OWN; ++i) {
+        cmin[i] = inf;
+        Z[i] = Nr[i] = 0.f;
     }
-    if (!in) return;
-    const size_t o = (size_t)gy * P.W + gx;
-    const bool ok = cmin < inf;
-    range[o] = ok ? Z / Nr : 0.f;
-    if (cost) cost[o] = ok ? cmin - P.T * logf(Z) : 0.f;
-    if (aux) {
-        aux[3 * o] = ok ? cmin : inf;
-        aux[3 * o + 1] = Z;
-        aux[3 * o + 2] = ok ? Nr / Z : 0.f;
+    for (int base = 0; base < P.K; base += ROUND) {
+        const int n = min(P.K - base, ROUND);
+        for (int k0 = 0; k0 < n; k0 += 2 * FG) {
+            // a group past the round's end repeats its last plane and stores nothing
+            const int k = k0 + 2 * group, np = max(0, min(2, n - k));
+            const PlaneD pl0 = P.planes[base + min(k, n - 1)], pl1 = P.planes[base + min(k + 1, n - 1)];
+            __syncthreads();  // the previous pairs' windows are done
+            warp_tile<G>(P, pl0, pl1, bx - RHO, by - RHO, tid, W2);
+            __syncthreads();
+            float2 best[PX];
+#pragma unroll
+            for (int i = 0; i < PX; ++i) best[i] = dup2(inf);
+            for (int j = 0; j < P.n_cams; ++j) {
+                float2 mb[PX], cov[PX], vb[PX];
+                pair_windows<G>(R, W2 + j * G::NPOS, lx, ly, ma, mb, cov, vb);
+#pragma unroll
+                for (int i = 0; i < PX; ++i) {
+                    const bool ok0 = !isnan(mb[i].x) && !(va[i] < lim || vb[i].x < lim);
+                    const bool ok1 = !isnan(mb[i].y) && !(va[i] < lim || vb[i].y < lim);
+                    const float2 s = sqrt_rn2(mul2(dup2(va[i]), vb[i])), z = div_rn2(cov[i], s, rcp_rn2(s));
+                    const float c0 = 0.5f * (1.0f - z.x), c1 = 0.5f * (1.0f - z.y);
+                    if (ok0 && c0 < best[i].x) best[i].x = c0;
+                    if (ok1 && c1 < best[i].y) best[i].y = c1;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < PX; ++i) {
+                float* c = Cs + k * NPIX + (ly + i) * SW + lx;
+                if (np > 0) c[0] = best[i].x;
+                if (np > 1) c[NPIX] = best[i].y;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < OWN; ++i) {
+            const int px = threadIdx.x + i * FG * ST;
+            if (px >= NPIX) continue;
+            const float4 ray = ray_at(P, bx + px % SW, by + px / SW);
+            for (int k = 0; k < n; ++k) {
+                const PlaneD pl = P.planes[base + k];
+                const float bq = Cs[k * NPIX + px];
+                const float rho_k = div_rn(plane_dot(pl, ray), pl.d, rcp_rn(pl.d));
+                // the smaller of the old minimum and bq becomes the new one; the
+                // other side's weight is exp(-|difference| / T), its own 1
+                const bool on = bq < inf, lt = on && bq < cmin[i];
+                const float x = lt ? cmin[i] - bq : bq - cmin[i];
+                const float f = x < inf ? __expf(-div_rn(x, P.T, inv_T)) : 0.f;
+                const float z = lt ? __fadd_rn(__fmul_rn(Z[i], f), 1.0f) : __fadd_rn(Z[i], f);
+                const float w = lt ? __fmaf_rn(1.0f, rho_k, __fmul_rn(Nr[i], f)) : __fmaf_rn(f, rho_k, Nr[i]);
+                Z[i] = on ? z : Z[i];
+                Nr[i] = on ? w : Nr[i];
+                cmin[i] = fminf(cmin[i], bq);
+            }
+        }
+        __syncthreads();  // the costs stay until they are read
+    }
+#pragma unroll
+    for (int i = 0; i < OWN; ++i) {
+        const int px = threadIdx.x + i * FG * ST;
+        const int gx = bx + px % SW, gy = by + px / SW;
+        if (px >= NPIX || gx >= P.W || gy >= P.H) continue;
+        const size_t o = (size_t)gy * P.W + gx;
+        const bool use = gx >= RHO && gy >= RHO && gx < P.W - RHO && gy < P.H - RHO && !isnan(P.rays[o].x);
+        const bool ok = use && cmin[i] < inf;
+        range[o] = ok ? Z[i] / Nr[i] : 0.f;
+        if (cost) cost[o] = ok ? cmin[i] - P.T * logf(Z[i]) : 0.f;
+        if (aux) {
+            aux[3 * o] = ok ? cmin[i] : inf;
+            aux[3 * o + 1] = use ? Z[i] : 0.f;
+            aux[3 * o + 2] = ok ? Nr[i] / Z[i] : 0.f;
+        }
     }
 }
 
@@ -345,72 +405,81 @@ struct GradOut {
     float* cam[PS_MAX_CAMS];
 };
 
-// Shared-memory layout of the backward kernel (floats), for window radius
-// RHO and nc matching cameras.  nf = 4 nc + 3 coefficient fields.
+// Shared memory of the backward kernel, in floats, for nc matching cameras
+// and nf = 4 nc + 3 coefficient fields (all of them pairs).
 template <int RHO>
 struct BwdLayout {
-    static constexpr int HW = DT + 2 * RHO, NPOS = HW * HW, BUF = HW * DS;
-    static constexpr int FS = DT + 1;  // field row stride
-    static constexpr int HS = HW + 1;  // horizontal-sum row stride (odd: the row-per-thread writes are conflict-free)
+    using G = Tile<RHO, 16, 1>;
+    static constexpr int FS = G::SW + 1;    // field row stride (pairs)
+    static constexpr int HS = G::HWC + 1;   // horizontal sums' row stride (pairs)
+    // odd strides: lanes on consecutive rows reach distinct banks
+    static_assert(FS % 2 == 1 && HS % 2 == 1, "conflict-free rows");
     __host__ __device__ static constexpr int nf(int nc) { return 4 * nc + 3; }
-    // Rs, gR, nc x (Ws, gW), chain data (8 floats + 1 cell per sample and
-    // camera), horizontal box sums [nf][DT][HS], fields / vertical box sums
-    // [nf][NPOS] (the fields [nf][DT][FS] are dead once the horizontal sums exist)
+    // warped pairs [nc][NPOS], fields [nf][TH][FS], horizontal sums [nf][TH][HS], reference [NPOS]
     __host__ __device__ static constexpr size_t floats(int nc) {
-        return (size_t)(2 + 2 * nc) * BUF + (size_t)nc * NPOS * 9 + (size_t)nf(nc) * DT * HS +
-               (size_t)nf(nc) * NPOS;
+        return 2 * ((size_t)nc * G::NPOS + (size_t)nf(nc) * G::TH * (FS + HS)) + G::NPOS;
     }
-    static_assert(NPOS >= DT * FS, "the vertical sums reuse the field storage");
 };
 
-// The sample of halo position (gx, gy) through plane P in camera C, with
-// what the chain rule needs later: the bilinear cell (y0 << 16 | x0, -1 when
-// invalid), its weights (ax, ay) and m = (X x g, g), g = J^T (dw/du, dw/dv),
-// J the 2 x 3 projection Jacobian at X (camera frame); gw m is then the
-// sample's contribution to the gradient of a left perturbation (w, v) of
-// ref_to_cam.  w is computed exactly as in the forward (warp_at).
-struct WarpJ {
-    float w;
-    int cell;
-    float ax, ay;
-    float m[6];
-};
-
-__device__ __forceinline__ WarpJ warp_jac(const DiffP& P, const DiffCam& C, const PlaneD& pl, int gx, int gy) {
-    WarpJ o;
-    const Warp wp = warp_at(P, C, pl, gx, gy);
-    o.w = wp.w;
-    o.cell = -1;
-    o.ax = o.ay = 0.f;
-#pragma unroll
-    for (int i = 0; i < 6; ++i) o.m[i] = 0.f;
-    if (isnan(wp.w)) return o;
-    const int Wc = C.c.width;
-    const int xa = (int)floorf(wp.u), ya = (int)floorf(wp.v);
-    const int xb = min(xa + 1, Wc - 1), yb = min(ya + 1, C.c.height - 1);
-    const float ax = wp.u - (float)xa, ay = wp.v - (float)ya;
+// Chain of one halo position's samples of both planes in one camera: gw =
+// dL/dw per plane goes to the image's four texels (global atomics, img may be
+// NULL); m receives (X x g, g) with g = J^T (dw/du, dw/dv), J the 2 x 3
+// projection Jacobian at X (camera frame): gw m is the samples' contribution
+// to the gradient of a left perturbation (w, v) of ref_to_cam.
+// The warp is the forward's; g comes from reverse-mode differentiation of the
+// projection: the adjoints of the distorted point, of the normalised point
+// (mx, my), then of X through mx = X / den, my = Y / den, den = xi |X| + Z.
+__device__ __forceinline__ void chain_pair(const DiffCam& C, const PlaneD& p0, const PlaneD& p1, const float4& r,
+                                           float2 gw, float* img, float2 (&m)[6]) {
+    const Proj o = project_pair(C, p0, p1, r);
+    Cell c[2];
+    cell_at(C, o.u.x, o.v.x, c[0]);
+    cell_at(C, o.u.y, o.v.y, c[1]);
+    float2 gu, gv;
     const float* I = C.img;
-    const float i00 = I[(size_t)ya * Wc + xa], i10 = I[(size_t)ya * Wc + xb];
-    const float i01 = I[(size_t)yb * Wc + xa], i11 = I[(size_t)yb * Wc + xb];
-    const float dwdu = (1.f - ay) * (i10 - i00) + ay * (i11 - i01);
-    const float dwdv = (1.f - ax) * (i01 - i00) + ax * (i11 - i10);
-    float g[3];
-    project_vjp_f(C.c, wp.X, wp.Y, wp.Z, dwdu, dwdv, g);
-    o.cell = (ya << 16) | xa;
-    o.ax = ax;
-    o.ay = ay;
-    o.m[0] = wp.Y * g[2] - wp.Z * g[1];
-    o.m[1] = wp.Z * g[0] - wp.X * g[2];
-    o.m[2] = wp.X * g[1] - wp.Y * g[0];
-    o.m[3] = g[0];
-    o.m[4] = g[1];
-    o.m[5] = g[2];
-    return o;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const float i00 = I[c[q].i00], i10 = I[c[q].i10], i01 = I[c[q].i01], i11 = I[c[q].i11];
+        const float ax = c[q].ax, ay = c[q].ay;
+        (q ? gu.y : gu.x) = __fmaf_rn(1.f - ay, i10 - i00, __fmul_rn(ay, i11 - i01));
+        (q ? gv.y : gv.x) = __fmaf_rn(1.f - ax, i01 - i00, __fmul_rn(ax, i11 - i10));
+    }
+    const float2 drad = fma2(C.k2x2, o.r2, C.k1);
+    // d(xd, yd)/d(mx, my) = [[a, b], [b, d]]
+    const float2 mx = o.mx, my = o.my, mx2 = add2(mx, mx), my2 = add2(my, my);
+    const float2 a = fma2(C.p2x6, mx, fma2(C.p1x2, my, fma2(mul2(mx2, mx), drad, o.rad)));
+    const float2 b = fma2(C.p2x2, my, fma2(mul2(mx2, my), drad, mul2(C.p1x2, mx)));
+    const float2 d = fma2(C.p2x2, mx, fma2(C.p1x6, my, fma2(mul2(my2, my), drad, o.rad)));
+    const float2 gxd = mul2(gu, C.fx), gyd = mul2(gv, C.fy);
+    const float2 gmx = fma2(gxd, a, mul2(gyd, b)), gmy = fma2(gxd, b, mul2(gyd, d));
+    const float2 gden = neg2(mul2(fma2(gmx, mx, mul2(gmy, my)), o.inv));  // dL/dden
+    const float2 xn = div_rn2(C.xi, o.n, rcp_rn2(o.n));                   // d(xi n)/dX = xi X / n
+    const float2 gx = mul2(gden, xn);
+    const float2 g0 = fma2(gmx, o.inv, mul2(gx, o.X)), g1 = fma2(gmy, o.inv, mul2(gx, o.Y));
+    const float2 g2 = mul2(gden, fma2(xn, o.Z, dup2(1.0f)));
+    m[0] = fma2(o.Y, g2, neg2(mul2(o.Z, g1)));
+    m[1] = fma2(o.Z, g0, neg2(mul2(o.X, g2)));
+    m[2] = fma2(o.X, g1, neg2(mul2(o.Y, g0)));
+    m[3] = g0;
+    m[4] = g1;
+    m[5] = g2;
+    if (img) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const float g = q ? gw.y : gw.x, ax = c[q].ax, ay = c[q].ay;
+            if (g == 0.f) continue;
+            if (!PS_DCHECK(c[q].i00 >= 0 && c[q].i11 < C.width * C.height, CHK_GATHER)) continue;
+            atomicAdd(&img[c[q].i00], g * (1.f - ax) * (1.f - ay));
+            atomicAdd(&img[c[q].i10], g * ax * (1.f - ay));
+            atomicAdd(&img[c[q].i01], g * (1.f - ax) * ay);
+            atomicAdd(&img[c[q].i11], g * ax * ay);
+        }
+    }
 }
 
-// Backward of the soft sweep for one 16 x 16 tile.  Per plane:
-//  1. warp the halo for every camera (samples + chain data, warp_jac);
-//  2. per pixel, the plane's cost and winning camera jb as in the forward,
+// Backward of the soft sweep for one 16 x 16 tile.  Per pair of planes:
+//  1. warp the halo for every camera, as in the forward;
+//  2. per pixel and plane, the cost and winning camera jb as in the forward,
 //     dL/dC, and the ZNCC gradient coefficients ka = gz / sqrt(va vb),
 //     kz_a = gz z / va, kz_b = gz z / vb (gz = dL/dZNCC);
 //  3. window gradients as box sums.  For a window sample q of pixel p,
@@ -425,224 +494,257 @@ __device__ __forceinline__ WarpJ warp_jac(const DiffP& P, const DiffCam& C, cons
 //     per-plane, per-camera centre (b), which leaves every difference
 //     unchanged and keeps the products small.  The box sums are separable
 //     (rows, then columns) in shared memory: no atomics;
-//  4. chain every sample with dL/dw != 0: dL/dI to its four texels (global
-//     atomics) and gw m to the pose accumulators.
+//  4. chain every sample with dL/dw != 0 (chain_pair: the warp of such a
+//     sample is computed again rather than kept from step 1).
 // After the planes: dL/dref of the halo (global atomics) and the CTA's pose
-// gradient (FP64 atomics).
-template <int RHO>
-__global__ void __launch_bounds__(DNT) soft_bwd_kernel(const __grid_constant__ DiffP P, const float* aux,
-                                                      const float* g_range, const float* g_cost, float* g_ref,
-                                                      const __grid_constant__ GradOut G, double* g_pose) {
+// gradient (FP64 atomics).  MC: most cameras (their pose accumulators are
+// registers).
+template <int RHO, int MC>
+__global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__ DiffP P, const float* aux,
+                                                         const float* g_range, const float* g_cost, float* g_ref,
+                                                         const __grid_constant__ GradOut GO, double* g_pose) {
     using BL = BwdLayout<RHO>;
-    constexpr int HW = BL::HW, NPOS = BL::NPOS, BUF = BL::BUF, FS = BL::FS, HS = BL::HS;
+    using G = typename BL::G;
+    constexpr int HWC = G::HWC, NPOS = G::NPOS, TH = G::TH, FS = BL::FS, HS = BL::HS, N = G::N, RPT = G::RPT, SW = G::SW;
+    constexpr int PX = 1;
     const int nc = P.n_cams, nf = BL::nf(nc);
-    extern __shared__ float sm[];
-    float* Rs = sm;                                   // reference
-    float* gR = Rs + BUF;                             // dL/dref, summed over planes
-    float* Ws = gR + BUF;                             // [nc] warped samples of the current plane
-    float* gW = Ws + nc * BUF;                        // [nc] dL/dw of the current plane
-    float* Cm = gW + nc * BUF;                        // [nc][8][NPOS] m[0..5], ax, ay
-    int* Cc = reinterpret_cast<int*>(Cm + nc * 8 * NPOS);  // [nc][NPOS] bilinear cell
-    float* Hx = reinterpret_cast<float*>(Cc + nc * NPOS);  // [nf][DT][HS] horizontal box sums
-    float* FV = Hx + nf * DT * HS;                    // [nf][DT][FS] fields, then [nf][NPOS] box sums
-    __shared__ float red[DNT / 32][6 * PS_MAX_CAMS];
-    const int tid = threadIdx.x, lx = tid % DT, ly = tid / DT;
-    const int x0 = blockIdx.x * DT - RHO, y0 = blockIdx.y * DT - RHO;
-    const int gx = blockIdx.x * DT + lx, gy = blockIdx.y * DT + ly;
-    for (int p = tid; p < NPOS; p += DNT) {
-        const int hx = p % HW, hy = p / HW, x = x0 + hx, y = y0 + hy;
-        Rs[hy * DS + hx] = (x >= 0 && y >= 0 && x < P.W && y < P.H) ? P.ref[(size_t)y * P.W + x] : 0.0f;
-        gR[hy * DS + hx] = 0.f;
-    }
-    const bool in = gx < P.W && gy < P.H;
-    const size_t o = in ? (size_t)gy * P.W + gx : 0;
-    float4 ray = in ? P.rays[o] : make_float4(0.f, 0.f, 0.f, 0.f);
+    extern __shared__ __align__(16) float sm[];
+    float2* W2 = reinterpret_cast<float2*>(sm);
+    float2* F = W2 + nc * NPOS;
+    float2* Hx = F + nf * TH * FS;
+    float* R = reinterpret_cast<float*>(Hx + nf * TH * HS);
+    __shared__ float red[ST / 32][6 * MC];
+    const int tid = threadIdx.x, lx = tid % SW, ly = tid / SW * PX;
+    const int bx = blockIdx.x * SW, by = blockIdx.y * TH, x0 = bx - RHO, y0 = by - RHO;
+    load_ref<G>(P, x0, y0, R);
+    __syncthreads();
+    float ma[PX], va[PX];
+    ref_windows<G>(R, lx, ly, ma, va);
     const float inf = __int_as_float(0x7f800000);
-    float cmin = inf, Z = 1.f, E = 0.f, gr = 0.f, gs = 0.f;
-    if (in) {
-        cmin = aux[3 * o];
-        Z = aux[3 * o + 1];
-        E = aux[3 * o + 2];
-        gr = g_range ? g_range[o] : 0.f;
-        gs = g_cost ? g_cost[o] : 0.f;
+    const float lim = (float)N * 1e-8f, inv_T = __frcp_rn(P.T);
+    float cmin[PX], Z[PX], E[PX], gE[PX], gs[PX];
+    bool use[PX];
+#pragma unroll
+    for (int i = 0; i < PX; ++i) {
+        const int gx = bx + lx, gy = by + ly + i;
+        const bool in = gx >= RHO && gy >= RHO && gx < P.W - RHO && gy < P.H - RHO;
+        const size_t o = in ? (size_t)gy * P.W + gx : 0;
+        cmin[i] = in ? aux[3 * o] : inf;
+        Z[i] = in ? aux[3 * o + 1] : 1.f;
+        E[i] = in ? aux[3 * o + 2] : 0.f;
+        const float gr = in && g_range ? g_range[o] : 0.f;
+        gs[i] = in && g_cost ? g_cost[o] : 0.f;
+        use[i] = in && !isnan(P.rays[o].x) && cmin[i] < inf && (gr != 0.f || gs[i] != 0.f);
+        gE[i] = use[i] ? -gr / (E[i] * E[i]) : 0.f;
     }
-    const bool use = in && gx >= RHO && gy >= RHO && gx < P.W - RHO && gy < P.H - RHO && !isnan(ray.x) &&
-                     cmin < inf && (gr != 0.f || gs != 0.f);
-    const float gE = use ? -gr / (E * E) : 0.f;
-    float pose_acc[6 * PS_MAX_CAMS];
+    float pose_acc[MC][6];
 #pragma unroll
-    for (int i = 0; i < 6 * PS_MAX_CAMS; ++i) pose_acc[i] = 0.f;
-    __syncthreads();
-    const int qc = (RHO + DT / 2) * DS + RHO + DT / 2;  // centre of the tile
-    const float ca = Rs[qc];
-    for (int k = 0; k < P.K; ++k) {
-        const PlaneD pl = P.planes[k];
-        __syncthreads();  // the previous plane's chain is done with gW and the chain data
-        // 1. samples and chain data of the halo
-        for (int p = tid; p < NPOS; p += DNT) {
-            const int hx = p % HW, hy = p / HW;
-            for (int j = 0; j < nc; ++j) {
-                const WarpJ wj = warp_jac(P, P.cams[j], pl, x0 + hx, y0 + hy);
-                Ws[j * BUF + hy * DS + hx] = wj.w;
-                float* cm = Cm + j * 8 * NPOS + p;
+    for (int j = 0; j < MC; ++j)
 #pragma unroll
-                for (int i = 0; i < 6; ++i) cm[i * NPOS] = wj.m[i];
-                cm[6 * NPOS] = wj.ax;
-                cm[7 * NPOS] = wj.ay;
-                Cc[j * NPOS + p] = wj.cell;
-            }
-        }
+        for (int i = 0; i < 6; ++i) pose_acc[j][i] = 0.f;
+    float gR[RPT];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) gR[i] = 0.f;
+    const int qc = (RHO + TH / 2) * HWC + RHO + SW / 2;  // centre of the tile
+    const float ca = R[qc];
+    for (int k = 0; k < P.K; k += 2) {
+        const int np = min(2, P.K - k);
+        const PlaneD pl0 = P.planes[k], pl1 = P.planes[k + np - 1];
+        __syncthreads();  // the previous pair's chain is done with the samples and sums
+        warp_tile<G>(P, pl0, pl1, x0, y0, tid, W2);
         __syncthreads();
-        // the per-camera centre of this plane's warped samples (a broadcast read)
+        // the per-camera centre of this pair's warped samples (a broadcast read)
         auto centre = [&](int j) {
-            const float c = Ws[j * BUF + qc];
-            return isnan(c) ? 0.f : c;
+            const float2 c = W2[j * NPOS + qc];
+            return make_float2(isnan(c.x) ? 0.f : c.x, isnan(c.y) ? 0.f : c.y);
         };
-        // 2. the pixel's cost for this plane (as in the forward), its camera and coefficients
-        float best = inf;
-        int jb = -1;
-        Zn zb;
-        for (int j = 0; use && j < nc; ++j) {
-            Zn zn;
-            if (window_zncc<RHO>(Rs, Ws + j * BUF, lx, ly, &zn)) {
-                float c = 0.5f * (1.0f - zn.z);
-                if (c < best) {
-                    best = c;
-                    jb = j;
-                    zb = zn;
-                }
+        // 2. cost, camera and coefficients
+        float best[PX][2], z[PX][2], mb[PX][2], vb[PX][2], sab[PX][2];
+        int jb[PX][2];
+#pragma unroll
+        for (int i = 0; i < PX; ++i)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                best[i][q] = inf;
+                z[i][q] = mb[i][q] = 0.f;
+                vb[i][q] = sab[i][q] = 1.f;
+                jb[i][q] = -1;
             }
+        for (int j = 0; j < nc; ++j) {
+            float2 m2[PX], c2[PX], v2[PX];
+            pair_windows<G>(R, W2 + j * NPOS, lx, ly, ma, m2, c2, v2);
+            float2 ss[PX], zz[PX];
+#pragma unroll
+            for (int i = 0; i < PX; ++i) {
+                ss[i] = sqrt_rn2(mul2(dup2(va[i]), v2[i]));
+                zz[i] = div_rn2(c2[i], ss[i], rcp_rn2(ss[i]));
+            }
+#pragma unroll
+            for (int i = 0; i < PX; ++i)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const float m = q ? m2[i].y : m2[i].x, v = q ? v2[i].y : v2[i].x;
+                    const bool ok = use[i] && q < np && !isnan(m) && !(va[i] < lim || v < lim);
+                    const float c = 0.5f * (1.0f - (q ? zz[i].y : zz[i].x));
+                    if (ok && c < best[i][q]) {
+                        best[i][q] = c;
+                        jb[i][q] = j;
+                        z[i][q] = q ? zz[i].y : zz[i].x;
+                        mb[i][q] = m;
+                        vb[i][q] = v;
+                        sab[i][q] = q ? ss[i].y : ss[i].x;
+                    }
+                }
         }
-        float ka = 0.f, kza = 0.f, kzb = 0.f, mac = 0.f, mbc = 0.f;
-        if (jb >= 0) {
-            const float s = __expf(-(best - cmin) / P.T) / Z;
-            const float rho_k = plane_dot(pl, ray) / pl.d;
-            const float gC = gE * (-s * (rho_k - E) / P.T) + gs * s;
-            const float gz = -0.5f * gC;
-            ka = gz / zb.sab;
-            kza = gz * zb.z / zb.va;
-            kzb = gz * zb.z / zb.vb;
-            mac = zb.ma - ca;
-            mbc = zb.mb - centre(jb);
-        }
-        {
-            float* F = FV + ly * FS + lx;
+#pragma unroll
+        for (int i = 0; i < PX; ++i) {
+            const float4 ray = P.rays[use[i] ? (size_t)(by + ly + i) * P.W + bx + lx : 0];
+            float ka[2], kza[2], kzb[2], mac = ma[i] - ca, mbc[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const PlaneD& pl = q == 0 ? pl0 : pl1;
+                const float2 cb = centre(max(jb[i][q], 0));
+                // (a square root or quotient of a window that is not used may be NaN)
+                const float ez = __expf(div_rn(-(best[i][q] - cmin[i]), P.T, inv_T));
+                const float s = div_rn(ez, Z[i], rcp_rn(Z[i]));
+                const float rho_k = div_rn(plane_dot(pl, ray), pl.d, rcp_rn(pl.d));
+                const float gC = gE[i] * div_rn(-s * (rho_k - E[i]), P.T, inv_T) + gs[i] * s;
+                const float gz = -0.5f * gC, gzz = gz * z[i][q];
+                const bool on = jb[i][q] >= 0;
+                ka[q] = on ? div_rn(gz, sab[i][q], rcp_rn(sab[i][q])) : 0.f;
+                kza[q] = on ? div_rn(gzz, va[i], rcp_rn(va[i])) : 0.f;
+                kzb[q] = on ? div_rn(gzz, vb[i][q], rcp_rn(vb[i][q])) : 0.f;
+                mbc[q] = on ? mb[i][q] - (q ? cb.y : cb.x) : 0.f;
+            }
+            float2* f = F + (ly + i) * FS + lx;
             for (int j = 0; j < nc; ++j) {
-                const bool mine = j == jb;
-                F[(4 * j + 0) * DT * FS] = mine ? ka : 0.f;
-                F[(4 * j + 1) * DT * FS] = mine ? ka * mac : 0.f;
-                F[(4 * j + 2) * DT * FS] = mine ? kzb : 0.f;
-                F[(4 * j + 3) * DT * FS] = mine ? kzb * mbc : 0.f;
+                const bool m0 = jb[i][0] == j, m1 = jb[i][1] == j;
+                f[(4 * j + 0) * TH * FS] = make_float2(m0 ? ka[0] : 0.f, m1 ? ka[1] : 0.f);
+                f[(4 * j + 1) * TH * FS] = make_float2(m0 ? ka[0] * mac : 0.f, m1 ? ka[1] * mac : 0.f);
+                f[(4 * j + 2) * TH * FS] = make_float2(m0 ? kzb[0] : 0.f, m1 ? kzb[1] : 0.f);
+                f[(4 * j + 3) * TH * FS] = make_float2(m0 ? kzb[0] * mbc[0] : 0.f, m1 ? kzb[1] * mbc[1] : 0.f);
             }
-            F[(4 * nc + 0) * DT * FS] = ka * mbc;
-            F[(4 * nc + 1) * DT * FS] = kza;
-            F[(4 * nc + 2) * DT * FS] = kza * mac;
+            f[(4 * nc + 0) * TH * FS] = make_float2(ka[0] * mbc[0], ka[1] * mbc[1]);
+            f[(4 * nc + 1) * TH * FS] = make_float2(kza[0], kza[1]);
+            f[(4 * nc + 2) * TH * FS] = make_float2(kza[0] * mac, kza[1] * mac);
         }
         __syncthreads();
-        // 3a. horizontal box sums: halo column c collects pixels c - 2 RHO .. c of the row.
-        // Direct sums, not running ones: coefficients of low-texture windows are
-        // large, and a running sum would leave their rounding residue where the
-        // exact sum is zero
-        for (int it = tid; it < nf * DT; it += DNT) {
-            const float* fr = FV + it * FS;
-            float* hr = Hx + it * HS;
-            float v[DT];
+        // 3a. horizontal box sums: halo column c collects pixels c - 2 RHO .. c of
+        // the row.  Direct sums, not running ones: coefficients of low-texture
+        // windows are large, and a running sum would leave their rounding residue
+        // where the exact sum is zero
+        constexpr int RO = (HWC + 3) / 4;  // outputs of an item
+        for (int it = tid; it < 4 * nf * TH; it += ST) {
+            const int part = it / (nf * TH), fr = it - part * (nf * TH);
+            const float2* in = F + fr * FS;
+            float2* out = Hx + fr * HS;
+            const int c0 = part * RO;
+            float2 v[RO + 2 * RHO];
 #pragma unroll
-            for (int x = 0; x < DT; ++x) v[x] = fr[x];
-#pragma unroll
-            for (int c = 0; c < HW; ++c) {
-                float acc = 0.f;
-#pragma unroll
-                for (int x = (c - 2 * RHO > 0 ? c - 2 * RHO : 0); x <= (c < DT - 1 ? c : DT - 1); ++x) acc += v[x];
-                hr[c] = acc;
+            for (int t = 0; t < RO + 2 * RHO; ++t) {
+                const int x = c0 - 2 * RHO + t;
+                v[t] = x >= 0 && x < SW ? in[x] : dup2(0.f);
             }
-        }
-        __syncthreads();
-        // 3b. vertical box sums: halo row r collects rows r - 2 RHO .. r
-        for (int it = tid; it < nf * HW; it += DNT) {
-            const int f = it / HW, c = it - f * HW;
-            const float* hc = Hx + f * DT * HS + c;
-            float* vc = FV + f * NPOS + c;
-            float v[DT];
 #pragma unroll
-            for (int y = 0; y < DT; ++y) v[y] = hc[y * HS];
+            for (int c = 0; c < RO; ++c) {
+                float2 s = v[c];
 #pragma unroll
-            for (int r = 0; r < HW; ++r) {
-                float acc = 0.f;
-#pragma unroll
-                for (int y = (r - 2 * RHO > 0 ? r - 2 * RHO : 0); y <= (r < DT - 1 ? r : DT - 1); ++y) acc += v[y];
-                vc[r * HW] = acc;
+                for (int t = 1; t <= 2 * RHO; ++t) s = add2(s, v[c + t]);
+                if (c0 + c < HWC) out[c0 + c] = s;
             }
         }
         __syncthreads();
-        // 3c. per halo sample: dL/dw of every camera and this plane's part of dL/dref
-        for (int p = tid; p < NPOS; p += DNT) {
-            const int hx = p % HW, hy = p / HW, q = hy * DS + hx;
-            const float* V = FV + p;
-            const float a = Rs[q] - ca;
-            float g = -V[(4 * nc + 0) * NPOS] - a * V[(4 * nc + 1) * NPOS] + V[(4 * nc + 2) * NPOS];
-            for (int j = 0; j < nc; ++j) {
-                const float A1 = V[(4 * j + 0) * NPOS], A2 = V[(4 * j + 1) * NPOS];
-                const float A3 = V[(4 * j + 2) * NPOS], A4 = V[(4 * j + 3) * NPOS];
-                const float bw = Ws[j * BUF + q];
-                float gw = 0.f;
-                if (!isnan(bw)) {  // an invalid sample is in no used window: all its sums are zero
-                    const float b = bw - centre(j);
-                    gw = a * A1 - A2 - b * A3 + A4;
-                    g += b * A1;
-                }
-                gW[j * BUF + q] = gw;
+        // 3b, 4. vertical box sums at this thread's halo positions, dL/dw and the chain.
+        // The pose accumulators take the first plane's samples of every position,
+        // then the second's: the order of one plane at a time
+        auto column = [&](int f, int p) {  // sum of field f over rows y - 2 RHO .. y at halo position p
+            const int y = p / HWC, x = p - y * HWC;
+            const float2* in = Hx + (f * TH + y - 2 * RHO) * HS + x;
+            float2 v[2 * RHO + 1];
+#pragma unroll
+            for (int t = 0; t <= 2 * RHO; ++t) v[t] = y - 2 * RHO + t >= 0 && y - 2 * RHO + t < TH ? in[t * HS] : dup2(0.f);
+            float2 s = v[0];
+#pragma unroll
+            for (int t = 1; t <= 2 * RHO; ++t) s = add2(s, v[t]);
+            return s;
+        };
+        float2 g[RPT];  // dL/dref of this pair
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+            const int p = tid + i * ST;
+            g[i] = dup2(0.f);
+            if (p < NPOS) {
+                const float a = R[p] - ca;
+                g[i] = add2(fma2(dup2(-a), column(4 * nc + 1, p), neg2(column(4 * nc, p))), column(4 * nc + 2, p));
             }
-            gR[q] += g;
         }
-        __syncthreads();
-        // 4. chain dL/dw of every warped halo sample to the image and the pose
-        for (int p = tid; p < NPOS; p += DNT) {
-            const int hx = p % HW, hy = p / HW;
 #pragma unroll
-            for (int j = 0; j < PS_MAX_CAMS; ++j) {
-                if (j >= nc) break;
-                const float gw = gW[j * BUF + hy * DS + hx];
-                const int cell = Cc[j * NPOS + p];
-                if (gw == 0.f || cell < 0) continue;
-                const float* cm = Cm + j * 8 * NPOS + p;
+        for (int j = 0; j < MC; ++j) {
+            if (j >= nc) break;
+            const float2 cb = centre(j);
+            float2 gw[RPT], m[RPT][6];
 #pragma unroll
-                for (int i = 0; i < 6; ++i) pose_acc[6 * j + i] = fmaf(gw, cm[i * NPOS], pose_acc[6 * j + i]);
-                if (G.cam[j]) {
-                    const DiffCam& C = P.cams[j];
-                    const int Wc = C.c.width, xa = cell & 0xffff, ya = cell >> 16;
-                    if (!PS_DCHECK(xa < Wc && ya < C.c.height, CHK_GATHER)) continue;
-                    const int xb = min(xa + 1, Wc - 1), yb = min(ya + 1, C.c.height - 1);
-                    const float ax = cm[6 * NPOS], ay = cm[7 * NPOS];
-                    float* Gj = G.cam[j];
-                    atomicAdd(&Gj[(size_t)ya * Wc + xa], gw * (1.f - ax) * (1.f - ay));
-                    atomicAdd(&Gj[(size_t)ya * Wc + xb], gw * ax * (1.f - ay));
-                    atomicAdd(&Gj[(size_t)yb * Wc + xa], gw * (1.f - ax) * ay);
-                    atomicAdd(&Gj[(size_t)yb * Wc + xb], gw * ax * ay);
+            for (int i = 0; i < RPT; ++i) {
+                const int p = tid + i * ST;
+                gw[i] = dup2(0.f);
+#pragma unroll
+                for (int t = 0; t < 6; ++t) m[i][t] = dup2(0.f);
+                if (p < NPOS) {
+                    const float a = R[p] - ca;
+                    const float2 w = W2[j * NPOS + p], b = add2(w, neg2(cb)), a1 = column(4 * j, p);
+                    float2 v = fma2(dup2(a), a1, neg2(column(4 * j + 1, p)));
+                    v = add2(fma2(neg2(b), column(4 * j + 2, p), v), column(4 * j + 3, p));
+                    const float2 gb = fma2(b, a1, g[i]);
+                    // an invalid sample is in no used window: all its sums are zero
+                    if (!isnan(w.x)) {
+                        gw[i].x = v.x;
+                        g[i].x = gb.x;
+                    }
+                    if (!isnan(w.y)) {
+                        gw[i].y = v.y;
+                        g[i].y = gb.y;
+                    }
+                    if (gw[i].x != 0.f || gw[i].y != 0.f)
+                        chain_pair(P.cams[j], pl0, pl1, ray_at(P, x0 + p % HWC, y0 + p / HWC), gw[i], GO.cam[j], m[i]);
                 }
             }
+            // (a plane with gw = 0 may hold a sample that does not project)
+#pragma unroll
+            for (int i = 0; i < RPT; ++i)
+                if (gw[i].x != 0.f)
+#pragma unroll
+                    for (int t = 0; t < 6; ++t) pose_acc[j][t] = fmaf(gw[i].x, m[i][t].x, pose_acc[j][t]);
+#pragma unroll
+            for (int i = 0; i < RPT; ++i)
+                if (gw[i].y != 0.f)
+#pragma unroll
+                    for (int t = 0; t < 6; ++t) pose_acc[j][t] = fmaf(gw[i].y, m[i][t].y, pose_acc[j][t]);
+        }
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) gR[i] = (gR[i] + g[i].x) + g[i].y;
+    }
+    if (g_ref) {
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+            const int p = tid + i * ST, x = x0 + p % HWC, y = y0 + p / HWC;
+            if (p < NPOS && gR[i] != 0.f && PS_DCHECK(x >= 0 && y >= 0 && x < P.W && y < P.H, CHK_PIXEL))
+                atomicAdd(&g_ref[(size_t)y * P.W + x], gR[i]);
         }
     }
-    __syncthreads();
-    if (g_ref)
-        for (int p = tid; p < NPOS; p += DNT) {
-            const int hx = p % HW, hy = p / HW;
-            float g = gR[hy * DS + hx];
-            if (g != 0.f && PS_DCHECK(x0 + hx >= 0 && y0 + hy >= 0 && x0 + hx < P.W && y0 + hy < P.H, CHK_PIXEL))
-                atomicAdd(&g_ref[(size_t)(y0 + hy) * P.W + (x0 + hx)], g);
-        }
     if (g_pose) {
         const int lane = tid & 31, wid = tid >> 5;
 #pragma unroll
-        for (int i = 0; i < 6 * PS_MAX_CAMS; ++i) {
-            float v = pose_acc[i];
-            for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-            if (lane == 0) red[wid][i] = v;
-        }
+        for (int j = 0; j < MC; ++j)
+#pragma unroll
+            for (int i = 0; i < 6; ++i) {
+                float v = pose_acc[j][i];
+                for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+                if (lane == 0) red[wid][6 * j + i] = v;
+            }
         __syncthreads();
-        if (tid < 6 * P.n_cams) {
+        if (tid < 6 * nc) {
             double s = 0.0;
-            for (int w = 0; w < DNT / 32; ++w) s += (double)red[w][tid];
+            for (int w = 0; w < ST / 32; ++w) s += (double)red[w][tid];
             atomicAdd(&g_pose[tid], s);
         }
     }
@@ -661,6 +763,7 @@ struct psdiff_s {
     double T = 0.05;
     float4* rays = nullptr;
     PlaneD* planes = nullptr;
+    int sms = 0;
 };
 
 namespace {
@@ -689,11 +792,59 @@ int fill_params(const psdiff_t* h, const float* const* images, const ps_pose* re
         PS_ARG(images[1 + j] != nullptr, "psdiff: images[%d] is NULL", 1 + j);
         for (int i = 0; i < 12; ++i)
             PS_ARG(std::isfinite(i < 9 ? ref_to_cam[j].R[i] : ref_to_cam[j].t[i - 9]), "psdiff: pose %d not finite", j);
-        for (int i = 0; i < 9; ++i) P.cams[j].R[i] = (float)ref_to_cam[j].R[i];
-        for (int i = 0; i < 3; ++i) P.cams[j].t[i] = (float)ref_to_cam[j].t[i];
-        P.cams[j].c = to_camf(h->cams[j]);
-        P.cams[j].img = images[1 + j];
+        DiffCam& D = P.cams[j];
+        const CamF c = to_camf(h->cams[j]);
+        auto two = [](float v) { return make_float2(v, v); };
+        for (int i = 0; i < 9; ++i) D.R2[i] = two((float)ref_to_cam[j].R[i]);
+        for (int i = 0; i < 3; ++i) D.t2[i] = two((float)ref_to_cam[j].t[i]);
+        D.xi = two(c.xi); D.fx = two(c.fx); D.fy = two(c.fy); D.cx = two(c.cx); D.cy = two(c.cy);
+        D.k1 = two(c.k1); D.k2 = two(c.k2); D.k2x2 = two(2.0f * c.k2);
+        D.p1 = two(c.p1); D.p1x2 = two(2.0f * c.p1); D.p1x6 = two(6.0f * c.p1);
+        D.p2 = two(c.p2); D.p2x2 = two(2.0f * c.p2); D.p2x6 = two(6.0f * c.p2);
+        D.lim = two(c.lim);
+        D.r2_max = c.r2_max;
+        D.width = c.width;
+        D.height = c.height;
+        D.img = images[1 + j];
     }
+    return PS_OK;
+}
+
+}  // namespace
+
+namespace {
+
+template <class G>
+int launch_fwd(const DiffP& P, float* range, float* cost, float* aux, cudaStream_t s) {
+    const size_t smem = sizeof(float) * (ROUND * ST * G::PX + (2 * FG * P.n_cams + 1) * G::NPOS);
+    auto* kernel = soft_fwd_kernel<G>;
+    PS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kernel<<<dim3((P.W + G::SW - 1) / G::SW, (P.H + G::TH - 1) / G::TH), FG * ST, smem, s>>>(P, range, cost, aux);
+    PS_CUDA(cudaGetLastError());
+    return PS_OK;
+}
+
+// Tiles of 32 x 16 pixels, two under each other per thread; images of too few
+// of them for the SMs take twice as many of 16 x 16.
+template <int RHO>
+int forward(const psdiff_t* h, const DiffP& P, float* range, float* cost, float* aux, cudaStream_t s) {
+    using Wide = Tile<RHO, 32, 2>;
+    const long long tiles = (long long)((P.W + Wide::SW - 1) / Wide::SW) * ((P.H + Wide::TH - 1) / Wide::TH);
+    return tiles >= h->sms ? launch_fwd<Wide>(P, range, cost, aux, s)
+                           : launch_fwd<Tile<RHO, 16, 1>>(P, range, cost, aux, s);
+}
+
+template <int RHO, int MC>
+int launch_bwd(const psdiff_t* h, const DiffP& P, const float* aux, const float* g_range, const float* g_cost, float* g_ref,
+               const GradOut& G, double* g_pose, cudaStream_t s) {
+    using T = typename BwdLayout<RHO>::G;
+    // at most 170 KB (window 9, 4 cameras)
+    const size_t smem = sizeof(float) * BwdLayout<RHO>::floats(P.n_cams);
+    auto* kernel = soft_bwd_kernel<RHO, MC>;
+    PS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kernel<<<dim3((P.W + T::SW - 1) / T::SW, (P.H + T::TH - 1) / T::TH), ST, smem, s>>>(P, aux, g_range, g_cost, g_ref, G,
+                                                                                       g_pose);
+    PS_CUDA(cudaGetLastError());
     return PS_OK;
 }
 
@@ -743,7 +894,10 @@ extern "C" int psdiff_create(const ps_diff_desc* d, psdiff_t** out) {
     h->K = (int)planes.size();
     h->T = d->temperature;
     const size_t npx = (size_t)d->ref.width * d->ref.height;
-    cudaError_t e = cudaMalloc(&h->rays, sizeof(float4) * npx);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaMalloc(&h->rays, sizeof(float4) * npx);
     if (e == cudaSuccess) e = cudaMalloc(&h->planes, sizeof(PlaneD) * planes.size());
     if (e == cudaSuccess)
         e = cudaMemcpy(h->planes, planes.data(), sizeof(PlaneD) * planes.size(), cudaMemcpyHostToDevice);
@@ -769,16 +923,10 @@ extern "C" int psdiff_forward(psdiff_t* h, const float* const* images, const ps_
     DiffP P;
     int st = fill_params(h, images, ref_to_cam, P);
     if (st) return st;
-    dim3 grid((P.W + DT - 1) / DT, (P.H + DT - 1) / DT);
     cudaStream_t s = (cudaStream_t)stream;
-    if (P.rho == 2)
-        soft_fwd_kernel<2><<<grid, DNT, 0, s>>>(P, range, cost, aux);
-    else if (P.rho == 3)
-        soft_fwd_kernel<3><<<grid, DNT, 0, s>>>(P, range, cost, aux);
-    else
-        soft_fwd_kernel<4><<<grid, DNT, 0, s>>>(P, range, cost, aux);
-    PS_CUDA(cudaGetLastError());
-    return PS_OK;
+    if (P.rho == 2) return forward<2>(h, P, range, cost, aux, s);
+    if (P.rho == 3) return forward<3>(h, P, range, cost, aux, s);
+    return forward<4>(h, P, range, cost, aux, s);
 }
 
 extern "C" int psdiff_backward(psdiff_t* h, const float* const* images, const ps_pose* ref_to_cam, const float* aux,
@@ -792,24 +940,10 @@ extern "C" int psdiff_backward(psdiff_t* h, const float* const* images, const ps
     float* g_ref = g_images ? g_images[0] : nullptr;
     GradOut G;
     for (int j = 0; j < PS_MAX_CAMS; ++j) G.cam[j] = (g_images && j < h->n_cams) ? g_images[1 + j] : nullptr;
-    // at most 202 KB (window 9, 4 cameras)
-    const size_t smem = sizeof(float) * (P.rho == 2   ? BwdLayout<2>::floats(P.n_cams)
-                                         : P.rho == 3 ? BwdLayout<3>::floats(P.n_cams)
-                                                      : BwdLayout<4>::floats(P.n_cams));
-    dim3 grid((P.W + 15) / 16, (P.H + 15) / 16);
     cudaStream_t s = (cudaStream_t)stream;
-    if (P.rho == 2) {
-        PS_CUDA(cudaFuncSetAttribute(soft_bwd_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        soft_bwd_kernel<2><<<grid, DNT, smem, s>>>(P, aux, g_range, g_cost, g_ref, G, g_pose);
-    } else if (P.rho == 3) {
-        PS_CUDA(cudaFuncSetAttribute(soft_bwd_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        soft_bwd_kernel<3><<<grid, DNT, smem, s>>>(P, aux, g_range, g_cost, g_ref, G, g_pose);
-    } else {
-        PS_CUDA(cudaFuncSetAttribute(soft_bwd_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        soft_bwd_kernel<4><<<grid, DNT, smem, s>>>(P, aux, g_range, g_cost, g_ref, G, g_pose);
-    }
-    PS_CUDA(cudaGetLastError());
-    return PS_OK;
+    auto go = h->n_cams <= 2 ? (P.rho == 2 ? launch_bwd<2, 2> : P.rho == 3 ? launch_bwd<3, 2> : launch_bwd<4, 2>)
+                             : (P.rho == 2 ? launch_bwd<2, 4> : P.rho == 3 ? launch_bwd<3, 4> : launch_bwd<4, 4>);
+    return go(h, P, aux, g_range, g_cost, g_ref, G, g_pose, s);
 }
 
 namespace ps {
