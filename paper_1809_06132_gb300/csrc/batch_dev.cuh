@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(NT, 1) batch_kernel(const __grid_constant__ Ba
     const int tid = threadIdx.x;
     if (tid == 0) atomicMin(A.t, global_ns());
     const uint32_t tmem = tm_alloc(&s_tmem);
+    int held = -1;  // level whose record and cameras are in shared memory
     for (;;) {
         if (tid == 0) {
             const int t = atomicAdd(A.head, 1);
@@ -171,12 +172,17 @@ __global__ void __launch_bounds__(NT, 1) batch_kernel(const __grid_constant__ Ba
         const JobIO& io = A.io[job];
         int* c = A.ctr + job * C_N;
         if (kind == Q_SWEEP) {
-            // the level record goes to shared memory (read all through the item)
-            const int* src = reinterpret_cast<const int*>(A.levels + job * PS_MAX_LEVELS + lvl);
-            int* dst = reinterpret_cast<int*>(&sL);
-            for (int i = tid; i < (int)(sizeof(LevelD) / sizeof(int)); i += NT) dst[i] = src[i];
-            __syncthreads();
-            sweep_item<TH, KP>(sL, J.image_half, idx, cams, smem, &s_flag, tmem);
+            // the level record goes to shared memory (read all through the item),
+            // unless the item before left it there
+            const bool staged = held == job * PS_MAX_LEVELS + lvl;
+            held = job * PS_MAX_LEVELS + lvl;
+            if (!staged) {
+                const int* src = reinterpret_cast<const int*>(A.levels + held);
+                int* dst = reinterpret_cast<int*>(&sL);
+                for (int i = tid; i < (int)(sizeof(LevelD) / sizeof(int)); i += NT) dst[i] = src[i];
+                __syncthreads();
+            }
+            sweep_item<TH, KP>(sL, J.image_half, idx, staged, cams, smem, &s_flag, tmem);
         } else if (kind == Q_REF || kind == Q_STATS) {
             const PrepD& P = J.prep[lvl];
             const int y0 = idx * PREP_ROWS, n = min(PREP_ROWS, P.Hl - y0) * P.Wl;

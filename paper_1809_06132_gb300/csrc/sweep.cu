@@ -244,16 +244,20 @@ __global__ void __launch_bounds__(NT, 1) sweep_kernel(const __grid_constant__ Sw
     __shared__ uint32_t s_tmem;
     const int total = P.lv[0].n_items + (P.n_levels > 1 ? P.lv[1].n_items : 0);
     const uint32_t tmem = tm_alloc(&s_tmem);
+    int staged = -1;  // level whose cameras are in shared memory
     for (;;) {
         if (threadIdx.x == 0) s_tile = atomicAdd(tile_counter, 1);
         __syncthreads();
         const int t = s_tile;
         __syncthreads();
         if (t >= total) break;
-        if (t < P.lv[0].n_items)
-            sweep_item<TH_SINGLE, KP_SINGLE>(P.lv[0], P.image_half, t, cams, smem, &s_flag, tmem);
+        const int level = t < P.lv[0].n_items ? 0 : 1;
+        if (level == 0)
+            sweep_item<TH_SINGLE, KP_SINGLE>(P.lv[0], P.image_half, t, staged == 0, cams, smem, &s_flag, tmem);
         else
-            sweep_item<TH_SINGLE, KP_SINGLE>(P.lv[1], P.image_half, t - P.lv[0].n_items, cams, smem, &s_flag, tmem);
+            sweep_item<TH_SINGLE, KP_SINGLE>(P.lv[1], P.image_half, t - P.lv[0].n_items, staged == 1, cams, smem, &s_flag,
+                                             tmem);
+        staged = level;
     }
     tm_free(tmem);
 }
@@ -366,6 +370,73 @@ int check_camera(const ps_camera& c, const char* what) {
     PS_ARG(std::isfinite(c.cx) && std::isfinite(c.cy), "%s: principal point not finite", what);
     PS_ARG(c.r2_max > 0, "%s: r2_max must be > 0", what);
     return PS_OK;
+}
+
+// Time of a list of work items on S workers that each take the next item when
+// done: n[0] items of cost c[0], then n[1] of cost c[1].
+double list_time(int S, const long long n[2], const double c[2]) {
+    const long long full = n[0] / S, rest = n[0] % S;  // `rest` workers take one item more
+    const double la = full * c[0], lb = la + (rest ? c[0] : 0.0);
+    if (n[1] == 0) return lb;
+    auto done = [&](double t) {
+        auto one = [&](double l) { return t > l ? (long long)((t - l) / c[1] + 1e-9) : 0; };
+        return (S - rest) * one(la) + rest * one(lb);
+    };
+    double lo = la, hi = lb + c[1] * (double)(n[1] / S + 1);
+    for (int i = 0; i < 40; ++i) {
+        const double mid = 0.5 * (lo + hi);
+        (done(mid) >= n[1] ? hi : lo) = mid;
+    }
+    return std::max(hi, lb);
+}
+
+// Planes per work item of each level.  A work item costs about STEP1 us per
+// pair of planes and lone matching camera, STEP2 per pair of planes and two
+// cameras, and ITEM for itself (camera staging, reference tile, direction
+// tables, chunk record): measured 3.0, 6.3 and 8.5 us.  Small images need
+// short items to reach every SM (160 x 128, 32 planes: 18 items of 32 planes
+// or 144 of 4), large ones long items and a last wave that is nearly full
+// (streets of 1280 x 1024: 64 planes in the crop 743 us against 758 with 32;
+// 1024 x 544 with four cameras: 899 against 955; 1003 x 751 with three: 1493
+// against 1554).  The split whose items, heavier level first, end earliest by
+// these costs is taken; of nearly equal ones the one with fewer items.  The
+// results do not depend on it.
+void choose_chunks(const ps_sweep_desc* d, int sms, int chunk[PS_MAX_LEVELS]) {
+    const double STEP1 = 3.0, STEP2 = 6.3, ITEM = 8.5;
+    const double pair = STEP2 * (d->n_cams / 2) + STEP1 * (d->n_cams % 2);
+    struct Split { int chunk; long long items; double cost; };
+    std::vector<Split> all[PS_MAX_LEVELS];
+    for (int l = 0; l < d->n_levels; ++l) {
+        const ps_level& L = d->levels[l];
+        int K = 0;
+        for (int s = 0; s < L.n_sets; ++s) K += L.sets[s].count;
+        const int W = L.kind == PS_LEVEL_DOWNSAMPLE ? d->ref.width / L.factor : L.crop_w;
+        const int H = L.kind == PS_LEVEL_DOWNSAMPLE ? d->ref.height / L.factor : L.crop_h;
+        const long long tiles = (long long)((W + TW - 1) / TW) * ((H + TH_SINGLE - 1) / TH_SINGLE);
+        const int most = 2 * PLANE_CHUNK;  // an item's plane offsets fit its table in shared memory
+        for (int m = (K + most - 1) / most; m <= (K + 3) / 4 || all[l].empty(); ++m) {
+            const int c = std::min(K, 2 * ((K + 2 * m - 1) / (2 * m)));  // whole pairs
+            if (!all[l].empty() && all[l].back().chunk == c) continue;
+            all[l].push_back({c, tiles * ((K + c - 1) / c), ITEM + pair * ((c + 1) / 2)});
+            if (tiles * m > 64LL * sms) break;  // shorter items only add their own cost
+        }
+    }
+    double best = -1.0;
+    for (const Split& a : all[0]) {
+        const int n1 = d->n_levels > 1 ? (int)all[1].size() : 1;
+        for (int i = 0; i < n1; ++i) {
+            const Split b = d->n_levels > 1 ? all[1][i] : Split{0, 0, 1.0};
+            const bool swap = b.items > 0 && b.cost > a.cost;
+            const long long n[2] = {swap ? b.items : a.items, swap ? a.items : b.items};
+            const double c[2] = {swap ? b.cost : a.cost, swap ? a.cost : b.cost};
+            const double t = list_time(sms, n, c);
+            if (best < 0 || t < 0.99 * best) {
+                best = t;
+                chunk[0] = a.chunk;
+                if (d->n_levels > 1) chunk[1] = b.chunk;
+            }
+        }
+    }
 }
 
 ps_camera scaled_camera(const ps_camera& c, int s) {
@@ -548,6 +619,12 @@ extern "C" int psweep_create(const ps_sweep_desc* d, psweep_t** out) {
             return e_ == cudaErrorMemoryAllocation ? PS_ERR_OOM : PS_ERR_CUDA; \
         }                                            \
     } while (0)
+    {
+        int dev = 0, sms = 0;
+        PS_TRY(cudaGetDevice(&dev));
+        PS_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        choose_chunks(d, sms, h->chunk);
+    }
     for (int l = 0; l < d->n_levels; ++l) {
         const ps_level& L = d->levels[l];
         h->levels[l] = L;
@@ -606,18 +683,7 @@ extern "C" int psweep_create(const ps_sweep_desc* d, psweep_t** out) {
         PS_TRY(cudaMalloc(&h->ref_img[l], sizeof(float) * (size_t)W * H));
         PS_TRY(cudaMalloc(&h->stats[l], sizeof(float2) * (size_t)W * H));
         {
-            // work items: tiles x chunks of at most PLANE_CHUNK planes, so that
-            // items of both levels cost about the same and balance across SMs;
-            // a level with at least 16 waves of items even at twice that takes
-            // chunks of up to 2 PLANE_CHUNK (half the per-item work: direction
-            // tables, reference tile, chunk records; the tail stays short)
             const int n_tiles = ((W + TW - 1) / TW) * ((H + TH_SINGLE - 1) / TH_SINGLE);
-            int dev = 0, sms = 0;
-            PS_TRY(cudaGetDevice(&dev));
-            PS_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-            const int c2 = balanced_chunk(h->n_planes[l], 2 * PLANE_CHUNK);
-            const long long items2 = (long long)n_tiles * ((h->n_planes[l] + c2 - 1) / c2);
-            h->chunk[l] = items2 >= 16LL * sms ? c2 : balanced_chunk(h->n_planes[l], PLANE_CHUNK);
             const int n_chunks = (h->n_planes[l] + h->chunk[l] - 1) / h->chunk[l];
             if (n_chunks > 1)
                 PS_TRY(cudaMalloc(&h->partial[l], sizeof(float) * 7 * TH_SINGLE * TW * (size_t)n_tiles * n_chunks));

@@ -15,7 +15,7 @@ constexpr int TW = 64;   // output tile width (pixels)
 constexpr int NT = 768;  // threads per CTA (one CTA per SM); all of them warp (phase A)
 constexpr int NTV = 512; // threads that own output pixels: phase V, winner-take-all, outputs
 constexpr int RUN = 4;   // outputs per horizontal run (phase H)
-constexpr int PLANE_CHUNK = 32;  // most planes one work item sweeps (default)
+constexpr int PLANE_CHUNK = 32;  // planes per work item of a batch (default); single sweeps: choose_chunks
 static_assert(NT / 32 >= TW / RUN, "phase H: one warp per run, one lane per halo row");
 // Tile height TH (output rows; 16 or 24) and KP (planes warped per camera
 // before the window sums, 1 or 2) are template parameters of the tile
@@ -874,7 +874,11 @@ __device__ __forceinline__ void tile_finished(const LevelD& L, bool finished) {
 
 // End of a work item whose tile has several plane chunks (its chunk record
 // is written): count it, and when it completes the tile, merge the chunks'
-// records in plane order into the tile's outputs (or records).
+// records in plane order into the tile's outputs (or records).  A thread's
+// pixels and four chunks at a time load together: the merge is a chain of L2
+// latencies, and with many short chunks it held the last items (160 x 128 x
+// 32 planes in chunks of 4: sweep kernel 56 -> 33 us, with the cameras staged
+// once per level instead of per item).
 template <int TH>
 __device__ inline void merge_chunks(const LevelD& L, int tile, int* s_flag) {
     constexpr int SEG = TH / 8;
@@ -894,27 +898,26 @@ __device__ inline void merge_chunks(const LevelD& L, int tile, int* s_flag) {
     if (*s_flag && tid < NTV) {
         __threadfence();
         const float* base = L.partial + (size_t)tile * L.n_chunks * 7 * (TH * TW);
-#pragma unroll 1
-        for (int i = 0; i < SEG; ++i) {
+#pragma unroll
+        for (int i = 0; i < SEG; ++i) {  // unrolled: the pixels' loads overlap
             const int gx = tx * TW + ox, gy = ty * TH + oy0 + i;
             const int px = (oy0 + i) * TW + ox;
-            // global winner (first chunk holding the lowest cost: ties keep the lowest plane)
+            // global winner (first chunk holding the lowest cost: ties keep the
+            // lowest plane) and the lowest cost of the other chunks, in one pass
             int wc = -1;
-            float b1 = inf;
+            float b1 = inf, b2 = inf, cm = inf, cp = inf;
+#pragma unroll 4
             for (int c = 0; c < L.n_chunks; ++c) {
-                float v = __ldcg(base + ((size_t)c * 7 + 0) * (TH * TW) + px);
-                if (v < b1) {
-                    b1 = v;
-                    wc = c;
-                }
+                const float v = __ldcg(base + ((size_t)c * 7 + 0) * (TH * TW) + px);
+                const bool lt = v < b1;
+                b2 = fminf(b2, lt ? b1 : v);
+                wc = lt ? c : wc;
+                b1 = lt ? v : b1;
             }
-            float b2 = inf, cm = inf, cp = inf;
             int k = -1;
             if (wc >= 0) {
                 const float* P = base + (size_t)wc * 7 * (TH * TW) + px;
-                b2 = __ldcg(P + 1 * (TH * TW));
-                for (int c = 0; c < L.n_chunks; ++c)
-                    if (c != wc) b2 = fminf(b2, __ldcg(base + ((size_t)c * 7 + 0) * (TH * TW) + px));
+                b2 = fminf(b2, __ldcg(P + 1 * (TH * TW)));
                 k = __float_as_int(__ldcg(P + 6 * (TH * TW)));
                 const int lo = L.k_begin + wc * L.chunk, hi = min(L.k_end, lo + L.chunk);
                 cm = k > lo ? __ldcg(P + 2 * (TH * TW))
@@ -922,6 +925,8 @@ __device__ inline void merge_chunks(const LevelD& L, int tile, int* s_flag) {
                 cp = k < hi - 1 ? __ldcg(P + 3 * (TH * TW))
                                 : (wc + 1 < L.n_chunks ? __ldcg(base + ((size_t)(wc + 1) * 7 + 4) * (TH * TW) + px)
                                                        : inf);
+            } else {
+                b2 = inf;
             }
             if (gx < L.W && gy < L.H) {
                 if (L.records) {
@@ -1227,12 +1232,13 @@ __device__ __forceinline__ void stage_cams(const LevelD& L, CamS* cams) {
     if (threadIdx.x < L.n_cams) cam_consts(L.cams[threadIdx.x], cams[threadIdx.x]);
 }
 
-// One work item of a level: stage the matching cameras in shared memory and
+// One work item of a level: stage the matching cameras in shared memory
+// (unless they are there from the item before: about 2 us of one thread) and
 // run the tile routine for the level's window radius and image storage.
 template <int TH, int KP>
-__device__ __forceinline__ void sweep_item(const LevelD& L, int half, int item, CamS* cams, unsigned char* smem,
-                                           int* s_flag, uint32_t tmem) {
-    stage_cams(L, cams);
+__device__ __forceinline__ void sweep_item(const LevelD& L, int half, int item, bool staged, CamS* cams,
+                                           unsigned char* smem, int* s_flag, uint32_t tmem) {
+    if (!staged) stage_cams(L, cams);  // uniform over the CTA
     __syncthreads();
     if (half) {
         switch (L.rho) {
