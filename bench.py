@@ -528,8 +528,8 @@ def run_ours(args):
         "e2e": {"value": world * args.steps / (pipe_ms / 1e3), "unit": UNIT, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h, "api": "ps_pipe_push x K + ps_pipe_flush (two frames in flight)",
                 "serial": world * args.steps / (e2e_ms / 1e3), "serial_api": "psweep_frame_host per frame"},
-        # one prep launch for every level (reference images, statistics, quads), the sweep, the merge; 4 TSDF stages
-        "gpu_launches": args.steps * (1 + 2 + 4),
+        # one prep launch for every level (reference images, statistics, quads), the sweep, the merge; 3 TSDF launches
+        "gpu_launches": args.steps * (1 + 2 + 3),
         "clocks": clk,
         "render_s": render_s,
     }
@@ -921,7 +921,7 @@ def run_ringloop(args):
             "ms_per_step": main_case["ms_per_frame"], "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f32", "data": "synthetic (true range maps of the ring, boxes masked)",
             "config": {"workload": wl.name, "voxel": 0.02, "mu": 0.1, "local_map": "60 x 3 x 60 m"},
-            "cases": out, "render_s": render_s, "gpu_launches": 4 * n}
+            "cases": out, "render_s": render_s, "gpu_launches": 3 * n}
     print(json.dumps(line))
     return 0
 
@@ -991,7 +991,7 @@ def run_sharded(args):
             "config": dict(workload_config(args, wl, nf, world),
                            parallelism=f"plane ranges x{world} + record all-gather; TSDF hash parts x{world}",
                            l2="not flushed (the exchange is part of the step)"),
-            "tsdf_status": st, "gpu_launches": args.steps * (2 + 1 + 2 + 4), "clocks": clocks.summary(t0, t1)}
+            "tsdf_status": st, "gpu_launches": args.steps * (2 + 1 + 2 + 3), "clocks": clocks.summary(t0, t1)}
     if rank == 0:
         print(json.dumps(line))
     if world > 1:
@@ -1062,7 +1062,7 @@ def run_ringloop_swept(args):
             "blocks": {"on_gpu_end": T.count(), "peak_on_gpu": max(peak, T.count()),
                        "swapped_to_host": host_blocks},
             "depth_valid_fraction": {"mean": statistics.mean(valid) if valid else None},
-            "status": st, "render_s": render_s, "gpu_launches": n * 7}
+            "status": st, "render_s": render_s, "gpu_launches": n * 6}
     print(json.dumps(line))
     return 0
 

@@ -376,8 +376,9 @@ void ps_pipe_destroy(ps_pipe_t* p);
  * events.  psweep_profile_read synchronises those events and returns the
  * summed milliseconds per stage (host double[3]) and the number of calls
  * recorded, then restarts the count.  tsdf_profile / tsdf_profile_read do
- * the same for tsdf_integrate with 4 stages: 0 depth maximum, 1 block
- * allocation, 2 visible-block list, 3 integration. */
+ * the same for tsdf_integrate with 4 stages: 0 depth maximum (dense grids;
+ * hashed maps take it in stage 1), 1 block allocation, 2 visible-block list,
+ * 3 integration. */
 int psweep_profile(psweep_t* h, int32_t capacity);
 int psweep_profile_read(psweep_t* h, double* stage_ms, int32_t* n_calls);
 int tsdf_profile(tsdf_t* t, int32_t capacity);

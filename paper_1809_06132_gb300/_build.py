@@ -18,7 +18,7 @@ LIB = os.path.join(BUILD, "libpsweep.so")
 BUILD_CHECK = os.path.join(HERE, "_build_check")
 LIB_CHECK = os.path.join(BUILD_CHECK, "libpsweep_check.so")
 SOURCES = ["common.cu", "sweep.cu", "tsdf.cu", "batch.cu", "batch_k16.cu", "batch_k24.cu", "pipe.cu", "diff.cu"]
-HEADERS = ["internal.cuh", "sweep_dev.cuh", "batch_dev.cuh"]
+HEADERS = ["internal.cuh", "pairs.cuh", "sweep_dev.cuh", "batch_dev.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include")]
 

@@ -65,39 +65,6 @@ struct DiffP {
     DiffCam cams[PS_MAX_CAMS];
 };
 
-// Correctly rounded reciprocals, quotients and square roots without the
-// branches of the general forms (which serialise the samples of a thread),
-// for pairs: from an approximation y0 of 1 / b, y = RN(y0 + y0 (1 - b y0)); a
-// quotient is q + (a - b q) y with q = RN(a y), a square root g + (a - g g) h
-// with g = RN(a y), h = y / 2, y an approximation of 1 / sqrt(a) (P. Markstein,
-// "Computation of elementary functions on the IBM RISC System/6000
-// processor", 1990).  Compared with __frcp_rn, __fsqrt_rn and __fdiv_rn: no
-// difference over every mantissa at 8 exponents, every mantissa at 71, and
-// 10^9 random quotients.  Operands are normal numbers; a zero or infinite
-// operand gives NaN, which every caller rejects like the infinity.
-__device__ __forceinline__ float2 rcp_rn2(float2 b) {
-    const float2 y = make_float2(rcp_ftz(b.x), rcp_ftz(b.y));
-    return fma2(y, fma2(neg2(b), y, dup2(1.0f)), y);
-}
-// a / b for y = rcp_rn2(b)
-__device__ __forceinline__ float2 div_rn2(float2 a, float2 b, float2 y) {
-    const float2 q = mul2(a, y);
-    return fma2(fma2(neg2(b), q, a), y, q);
-}
-__device__ __forceinline__ float2 sqrt_rn2(float2 a) {
-    const float2 y = make_float2(rsqrt_ftz(a.x), rsqrt_ftz(a.y));
-    const float2 g = mul2(a, y);
-    return fma2(fma2(neg2(g), g, a), mul2(y, dup2(0.5f)), g);
-}
-__device__ __forceinline__ float rcp_rn(float b) {
-    const float y = rcp_ftz(b);
-    return __fmaf_rn(y, __fmaf_rn(-b, y, 1.0f), y);
-}
-__device__ __forceinline__ float div_rn(float a, float b, float y) {
-    const float q = __fmul_rn(a, y);
-    return __fmaf_rn(__fmaf_rn(-b, q, a), y, q);
-}
-
 // n . r of a plane and a ray.  The plane's offset along the ray, and the
 // bilinear blend below, are written with explicit roundings so that every
 // kernel computes the same samples (the costs decide integers: a camera, a

@@ -8,6 +8,7 @@
 #include <cuda_fp16.h>
 
 #include "internal.cuh"
+#include "pairs.cuh"
 
 namespace ps {
 
@@ -195,27 +196,6 @@ __device__ __forceinline__ float2 stats_px(const float* ref, int W, int H, int r
 }
 
 // ------------------------------------------------------------- sweep
-
-// Reciprocal and reciprocal square root as the single approximate PTX
-// instructions with subnormals flushed (rcp.approx.ftz, rsqrt.approx.ftz).
-// Their operands here (squared norms of points in metres, the unified
-// model's denominator, window variances above N 1e-8) are never subnormal,
-// where the non-flushing forms would add a rescaling sequence per call.
-__device__ __forceinline__ float rcp_ftz(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float rsqrt_ftz(float x) {
-    float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
 // Bilinear sample of a matching camera at pixel (u, v), as a centred
 // intensity; NaN when `ok` is false (the point does not project) or (u, v)
@@ -506,8 +486,6 @@ struct Geo {
     static_assert(HWL <= WS && 4 * NV + TW - RUN <= WS, "row stride covers the runs' loads");
     static_assert(HWL <= WS2 && 2 * NV2 + TW - RUN <= WS2, "pair row stride covers the runs' loads");
 };
-
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
 // Phases A, H and V of one matching camera for two planes at once (planes
 // at offsets d0 and d1 of the current set), on packed FP32 pairs: lane x is
