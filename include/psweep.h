@@ -570,6 +570,15 @@ int tsdf_dense_fuse_backward(const float* voxels_in, const int32_t* dims, const 
                              const ps_pose* world_to_cam, const float* g_D_out, float* g_D_in, float* g_depth,
                              double* g_pose, void* stream);
 
+/* The same gradient for a whole grid: g_out and g_in are {D, w} pairs like
+ * voxels_in (8-byte aligned; the weights' part of g_out is not read, that of
+ * g_in is written as zero), and g_depth and g_pose (either may be NULL) are
+ * WRITTEN, not added to.  Asynchronous on `stream`; allocates nothing. */
+int tsdf_dense_fuse_backward_grid(const float* voxels_in, const int32_t* dims, const double* origin, double voxel_size,
+                                  double mu, double w_max, const float* depth, const ps_camera* cam,
+                                  const ps_pose* world_to_cam, const float* g_out, float* g_in, float* g_depth,
+                                  double* g_pose, void* stream);
+
 /* Checked build (libpsweep_check.so, compiled with -DPS_CHECK; there is no
  * sanitizer on every machine this runs on): the kernels test the accesses
  * whose addresses come from data (image gathers at projected coordinates,

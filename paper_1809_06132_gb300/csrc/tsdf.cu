@@ -1091,7 +1091,10 @@ int dense_frame(const double* origin, double voxel_size, double mu, double w_max
 // observed voxels (g elsewhere); observed voxels with eta < mu add
 // g / (mu (w + 1)) to their pixel's depth gradient and -that * X_c / |X_c|
 // to X_c, which a left perturbation (w, v) of world_to_cam moves by
-// w x X_c + v (CTA reduction, FP64 atomics).
+// w x X_c + v (CTA reduction, FP64 atomics).  PAIRS: gD and gD_in are {D, w}
+// pairs like the voxels (weights get a zero gradient), so that a gradient of
+// the whole grid needs no pass that picks or places its D.
+template <bool PAIRS>
 __global__ void __launch_bounds__(256) dense_fuse_bwd_kernel(const __grid_constant__ FrameP F, int nbx, int nby,
                                                             int nbz, const float2* vox_in, const float* depth,
                                                             const float* gD, float* gD_in, float* g_depth,
@@ -1104,7 +1107,7 @@ __global__ void __launch_bounds__(256) dense_fuse_bwd_kernel(const __grid_consta
         const int v = (int)(i % B3);
         const int gx = (int)(b % nbx) * B + (v & 7), gy = (int)((b / nbx) % nby) * B + ((v >> 3) & 7),
                   gz = (int)(b / ((long long)nbx * nby)) * B + (v >> 6);
-        const float g = gD[i];
+        const float g = PAIRS ? reinterpret_cast<const float2*>(gD)[i].x : gD[i];
         float out = g;
         float eta, Xc[3];
         size_t pix;
@@ -1124,7 +1127,8 @@ __global__ void __launch_bounds__(256) dense_fuse_bwd_kernel(const __grid_consta
                 acc[5] += gx3[2];
             }
         }
-        if (gD_in) gD_in[i] = out;
+        if constexpr (PAIRS) reinterpret_cast<float2*>(gD_in)[i] = make_float2(out, 0.f);
+        else if (gD_in) gD_in[i] = out;
     }
     if (!g_pose) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1197,10 +1201,13 @@ extern "C" int tsdf_integrate_dense_static(float* voxels, const int32_t* dims, c
     return PS_OK;
 }
 
-extern "C" int tsdf_dense_fuse_backward(const float* voxels_in, const int32_t* dims, const double* origin,
-                                        double voxel_size, double mu, double w_max, const float* depth,
-                                        const ps_camera* cam, const ps_pose* w2c, const float* g_D_out,
-                                        float* g_D_in, float* g_depth, double* g_pose, void* stream) {
+namespace {
+
+// Both forms of the backward call: pairs = gradients of {D, w} pairs, and
+// g_depth and g_pose are cleared first.
+int dense_backward(const float* voxels_in, const int32_t* dims, const double* origin, double voxel_size, double mu,
+                   double w_max, const float* depth, const ps_camera* cam, const ps_pose* w2c, const float* g_D_out,
+                   float* g_D_in, float* g_depth, double* g_pose, bool pairs, void* stream) {
     clear_error();
     PS_ARG(voxels_in && dims && origin && depth && cam && w2c && g_D_out, "tsdf_dense_fuse_backward: NULL argument");
     PS_ARG(voxel_size > 0 && mu > 0 && w_max >= 1, "tsdf_dense_fuse_backward: need voxel_size > 0, mu > 0, w_max >= 1");
@@ -1218,11 +1225,36 @@ extern "C" int tsdf_dense_fuse_backward(const float* voxels_in, const int32_t* d
     PS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const long long n = (long long)dims[0] * dims[1] * dims[2];
     const int grid = (int)std::min<long long>((n + 255) / 256, (long long)sms * 8);
-    dense_fuse_bwd_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(F, dims[0] / 8, dims[1] / 8, dims[2] / 8,
-                                                                 reinterpret_cast<const float2*>(voxels_in), depth,
-                                                                 g_D_out, g_D_in, g_depth, g_pose);
+    cudaStream_t s = (cudaStream_t)stream;
+    if (pairs) {
+        if (g_depth) PS_CUDA(cudaMemsetAsync(g_depth, 0, sizeof(float) * (size_t)cam->width * cam->height, s));
+        if (g_pose) PS_CUDA(cudaMemsetAsync(g_pose, 0, 6 * sizeof(double), s));
+    }
+    auto* kernel = pairs ? dense_fuse_bwd_kernel<true> : dense_fuse_bwd_kernel<false>;
+    kernel<<<grid, 256, 0, s>>>(F, dims[0] / 8, dims[1] / 8, dims[2] / 8, reinterpret_cast<const float2*>(voxels_in),
+                                depth, g_D_out, g_D_in, g_depth, g_pose);
     PS_CUDA(cudaGetLastError());
     return PS_OK;
+}
+
+}  // namespace
+
+extern "C" int tsdf_dense_fuse_backward(const float* voxels_in, const int32_t* dims, const double* origin,
+                                        double voxel_size, double mu, double w_max, const float* depth,
+                                        const ps_camera* cam, const ps_pose* w2c, const float* g_D_out,
+                                        float* g_D_in, float* g_depth, double* g_pose, void* stream) {
+    return dense_backward(voxels_in, dims, origin, voxel_size, mu, w_max, depth, cam, w2c, g_D_out, g_D_in, g_depth,
+                          g_pose, false, stream);
+}
+
+extern "C" int tsdf_dense_fuse_backward_grid(const float* voxels_in, const int32_t* dims, const double* origin,
+                                             double voxel_size, double mu, double w_max, const float* depth,
+                                             const ps_camera* cam, const ps_pose* w2c, const float* g_out, float* g_in,
+                                             float* g_depth, double* g_pose, void* stream) {
+    clear_error();
+    PS_ARG(g_in != nullptr, "tsdf_dense_fuse_backward_grid: NULL argument");
+    return dense_backward(voxels_in, dims, origin, voxel_size, mu, w_max, depth, cam, w2c, g_out, g_in, g_depth, g_pose,
+                          true, stream);
 }
 
 namespace ps {

@@ -30,7 +30,7 @@ EXPORTS = ["psweep_create", "psweep_depth", "psweep_destroy", "tsdf_create", "ts
            "tsdf_swap_out", "tsdf_load", "tsdf_extract_points", "psbatch_create", "psbatch_run", "psbatch_timing", "psbatch_status",
            "psbatch_queue_stats", "psbatch_destroy", "psbatch_autotune", "ps_pipe_create", "ps_pipe_push",
            "ps_pipe_flush", "ps_pipe_destroy", "psdiff_create", "psdiff_forward", "psdiff_backward",
-           "psdiff_destroy", "tsdf_dense_fuse_backward",
+           "psdiff_destroy", "tsdf_dense_fuse_backward", "tsdf_dense_fuse_backward_grid",
            "ps_check_read", "ps_last_error", "ps_version", "ps_sync_status", "psweep_depth_planes",
            "psweep_merge_records", "tsdf_set_partition", "psweep_level_outputs"]
 MAX_PARTS = 16
@@ -167,6 +167,7 @@ def load(build_if_missing: bool = True):
     L.psdiff_destroy.restype = None
     L.tsdf_dense_fuse_backward.argtypes = [P, P, P, C.c_double, C.c_double, C.c_double, P, C.POINTER(ps_camera),
                                            C.POINTER(ps_pose), P, P, P, P, P]
+    L.tsdf_dense_fuse_backward_grid.argtypes = L.tsdf_dense_fuse_backward.argtypes
     L.ps_check_read.argtypes = [C.POINTER(C.c_uint32)]
     L.ps_sync_status.argtypes = [P, P]
     L.psweep_depth_planes.argtypes = [P, P, P, P, P, P]
@@ -196,14 +197,11 @@ def camera(c) -> ps_camera:
 
 
 def pose(p) -> ps_pose:
-    o = ps_pose()
-    R = np.asarray(p.R, dtype=np.float64).reshape(-1)
-    t = np.asarray(p.t, dtype=np.float64).reshape(-1)
-    for i in range(9):
-        o.R[i] = R[i]
-    for i in range(3):
-        o.t[i] = t[i]
-    return o
+    # one copy of the struct's 12 doubles: filling it element by element took 8 us a pose
+    a = np.empty(12)
+    a[:9] = np.asarray(p.R, dtype=np.float64).reshape(-1)[:9]
+    a[9:] = np.asarray(p.t, dtype=np.float64).reshape(-1)[:3]
+    return ps_pose.from_buffer_copy(a)
 
 
 def level(lv) -> ps_level:
@@ -223,10 +221,9 @@ def level(lv) -> ps_level:
 def boxes_array(boxes):
     b = np.zeros((0, 4), dtype=np.int32) if boxes is None else np.ascontiguousarray(boxes, dtype=np.int32)
     n = len(b)
-    arr = (ps_box * max(1, n))()
-    for i in range(n):
-        arr[i] = ps_box(*[int(v) for v in b[i]])
-    return arr, n
+    if n and (b.ndim != 2 or b.shape[1] != 4):
+        raise ValueError(f"boxes must be (n, 4) integers, got {b.shape}")
+    return ((ps_box * n).from_buffer_copy(b) if n else (ps_box * 1)()), n
 
 
 def _cuda_device(device, name: str):
@@ -720,22 +717,29 @@ def version() -> str:
 
 # ----------------------------------------------------------------- differentiable forms
 
+class _Pose:
+    """Rigid transform (R, t)."""
+    __slots__ = ("R", "t")
+
+    def __init__(self, R, t):
+        self.R, self.t = R, t
+
+
 def se3_exp_left(xi, p):
     """exp([w]x, v) applied on the left of pose p (R, t): rotation Exp(w) R,
     translation Exp(w) t + v; xi = (w, v)."""
     xi = np.asarray(xi, dtype=np.float64).reshape(6)
     w, v = xi[:3], xi[3:]
-    th = float(np.linalg.norm(w))
-    K = np.array([[0, -w[2], w[1]], [w[2], 0, -w[0]], [-w[1], w[0], 0]])
-    Rw = np.eye(3) if th == 0.0 else np.eye(3) + np.sin(th) / th * K + (1 - np.cos(th)) / th ** 2 * K @ K
     R = np.asarray(p.R, dtype=np.float64).reshape(3, 3)
     t = np.asarray(p.t, dtype=np.float64).reshape(3)
-
-    class _P:
-        pass
-    o = _P()
-    o.R, o.t = Rw @ R, Rw @ t + v
-    return o
+    if not w.any():   # no rotation, as in every gradient evaluated at delta = 0: R and t + v exactly
+        return _Pose(R.copy(), t + v)
+    th = float(np.linalg.norm(w))
+    if th == 0.0:
+        return _Pose(R.copy(), t + v)
+    K = np.array([[0, -w[2], w[1]], [w[2], 0, -w[0]], [-w[1], w[0], 0]])
+    Rw = np.eye(3) + np.sin(th) / th * K + (1 - np.cos(th)) / th ** 2 * K @ K
+    return _Pose(Rw @ R, Rw @ t + v)
 
 
 class SoftSweep:
@@ -784,7 +788,11 @@ class SoftSweep:
     def backward(self, images, poses, aux, g_range=None, g_cost=None, stream=None):
         """(per-image gradients, (n_cams, 6) float64 pose gradients (w, v))."""
         ims, ps = self._args(images, poses)
-        gi = [torch.zeros_like(im) for im in images]
+        if all(im.shape == images[0].shape for im in images):   # one buffer, cleared in one launch
+            gi = list(torch.zeros((len(images),) + tuple(images[0].shape), dtype=torch.float32,
+                                  device=images[0].device).unbind(0))
+        else:
+            gi = [torch.zeros_like(im) for im in images]
         gptr = (C.c_void_p * len(gi))(*[g.data_ptr() for g in gi])
         gp = torch.zeros((len(self.rig.cams), 6), dtype=torch.float64, device=images[0].device)
         gr = _dev(g_range.contiguous(), torch.float32, "g_range") if g_range is not None else None
@@ -860,10 +868,19 @@ class _DenseFuseFn(torch.autograd.Function):
     def backward(ctx, g_out):
         vin, dep = ctx.saved_tensors
         dims, origin, vs, mu, w_max, cam = ctx.grid
-        gin, gd, gp = tsdf_dense_fuse_backward(vin, dims, origin, vs, mu, w_max, dep, cam, ctx.pose,
-                                               g_out[..., 0])
-        g_vox = torch.zeros_like(vin)
-        g_vox[..., 0] = gin            # weights are observation counts: no gradient
+        # the kernel reads and writes {D, w} pairs: no gradient of its D is cut out
+        # of the grid's or put back into one of zeros (weights carry no gradient)
+        g = g_out.contiguous()
+        if g.data_ptr() % 8:   # a view that starts between pairs
+            g = g.clone()
+        g_vox, gd = torch.empty_like(vin), torch.empty_like(dep)
+        gp = torch.empty(6, dtype=torch.float64, device=dep.device)
+        d = (C.c_int32 * 3)(*[int(v) for v in dims])
+        o = (C.c_double * 3)(*[float(v) for v in origin])
+        _check(load().tsdf_dense_fuse_backward_grid(
+            _dev(vin, torch.float32, "voxels_in"), d, o, float(vs), float(mu), float(w_max),
+            _dev(dep, torch.float32, "depth"), C.byref(camera(cam)), C.byref(pose(ctx.pose)),
+            _dev(g, torch.float32, "g_out"), g_vox.data_ptr(), gd.data_ptr(), gp.data_ptr(), _stream_ptr(None)))
         dt, dev = ctx.delta_meta
         return None, None, gp.to(dtype=dt, device=dev), g_vox, gd
 
