@@ -1248,7 +1248,7 @@ struct MergeP {
     int W, H;
     const float* low;
     const float *low_c1, *low_c2;
-    int s, Wl, Hl;
+    int s, shift, Wl, Hl;           // downsampling factor s = 1 << shift
     const float* crop;
     const float *crop_c1, *crop_c2;
     int cx0, cy0, cw, ch;
@@ -1270,21 +1270,27 @@ __device__ __forceinline__ bool keep_level(const MergeP& P, float c1, float c2, 
 // where the crop covers (u, v) and has a depth; with the cost filters on, a
 // level pixel that fails them contributes nothing.
 __device__ __forceinline__ float merge_px(const MergeP& P, int u, int v) {
-    float val = 0.f;
+    // every load is issued before the first result is needed
+    float dl = 0.f, l1 = 0.f, l2 = 0.f, dc = 0.f, c1 = 0.f, c2 = 0.f;
+    const int lv = min(v >> P.shift, P.Hl - 1);
     if (P.low) {
-        int lu = min(u / P.s, P.Wl - 1), lv = min(v / P.s, P.Hl - 1);
-        size_t i = (size_t)lv * P.Wl + lu;
-        val = P.low[i];
-        if (P.filter && val > 0.f &&
-            !keep_level(P, P.low_c1[i], P.low_c2[i], (float)(P.s * lv) + 0.5f * (float)(P.s - 1)))
-            val = 0.f;
+        const size_t i = (size_t)lv * P.Wl + min(u >> P.shift, P.Wl - 1);
+        dl = P.low[i];
+        if (P.filter) {
+            l1 = P.low_c1[i];
+            l2 = P.low_c2[i];
+        }
     }
     if (P.crop && u >= P.cx0 && u < P.cx0 + P.cw && v >= P.cy0 && v < P.cy0 + P.ch) {
-        size_t i = (size_t)(v - P.cy0) * P.cw + (u - P.cx0);
-        float c = P.crop[i];
-        if (c > 0.f && (!P.filter || keep_level(P, P.crop_c1[i], P.crop_c2[i], (float)v))) val = c;
+        const size_t i = (size_t)(v - P.cy0) * P.cw + (u - P.cx0);
+        dc = P.crop[i];
+        if (P.filter) {
+            c1 = P.crop_c1[i];
+            c2 = P.crop_c2[i];
+        }
     }
-    return val;
+    if (P.filter && dl > 0.f && !keep_level(P, l1, l2, (float)(P.s * lv) + 0.5f * (float)(P.s - 1))) dl = 0.f;
+    return dc > 0.f && (!P.filter || keep_level(P, c1, c2, (float)v)) ? dc : dl;
 }
 
 // Local depth continuity at (u, v) of the merged map: the pixel keeps its
