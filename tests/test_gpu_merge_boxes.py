@@ -36,4 +36,6 @@ def test_boxes_mask_the_merged_map(window, n):
     for x0, y0, x1, y1 in b:
         keep[max(y0, 0):max(y1, 0), max(x0, 0):max(x1, 0)] = False
     want = torch.where(torch.from_numpy(keep).cuda(), plain, torch.zeros_like(plain))
-    assert torch.equal(sw.depth(ims, boxes=b), want) and (plain > 0).sum() > 500
+    assert torch.equal(sw.depth(ims, boxes=b), want)
+    # a window of one pixel has no neighbours to agree with: it keeps nothing
+    assert (plain > 0).sum() > 500 if window != 1 else not plain.any()
