@@ -25,7 +25,8 @@
 //                    ref_to_cam pose (CTA reduction, FP64 atomics).
 // Both are bound by instruction issue and latency (DRAM holds the images and
 // ray table once).  A forward and backward pass through autograd, 640 x 512,
-// 128 planes, 2 cameras: 5964 -> 4233 us; 96 x 80, 32 planes: 689 -> 597 us.
+// 128 planes, 2 cameras: 5.89 -> 4.09 ms (device time of the backward kernel
+// 4.22 -> 2.78 ms); 96 x 80, 32 planes: 672 -> 523 us.
 // Before: one pixel per thread, general divisions and square roots (their
 // slow-path branches serialise a thread's samples), the reference window's
 // sums repeated per plane, and a backward of one plane at a time with seven
@@ -163,6 +164,9 @@ struct Tile {
     static constexpr int HWC = SW + 2 * RHO, HH = TH + 2 * RHO, NPOS = HWC * HH;
     static constexpr int RPT = (NPOS + ST - 1) / ST;       // halo positions per thread
     static constexpr int N = (2 * RHO + 1) * (2 * RHO + 1);
+    // row stride of the reference samples: 16 mod 32 where a warp covers two
+    // rows of 16, so that they reach distinct banks
+    static constexpr int RS = SW == 16 ? 48 : HWC;
 };
 
 // Mean and sum of squared deviations of the reference windows of a thread's
@@ -176,13 +180,13 @@ __device__ __forceinline__ void ref_windows(const float* R, int lx, int ly, floa
         float s = 0.f;
         for (int dy = 0; dy <= 2 * RHO; ++dy)
 #pragma unroll
-            for (int dx = 0; dx <= 2 * RHO; ++dx) s += R[(ly + i + dy) * G::HWC + lx + dx];
+            for (int dx = 0; dx <= 2 * RHO; ++dx) s += R[(ly + i + dy) * G::RS + lx + dx];
         const float m = s / (float)G::N;
         float v = 0.f;
         for (int dy = 0; dy <= 2 * RHO; ++dy)
 #pragma unroll
             for (int dx = 0; dx <= 2 * RHO; ++dx) {
-                const float e = R[(ly + i + dy) * G::HWC + lx + dx] - m;
+                const float e = R[(ly + i + dy) * G::RS + lx + dx] - m;
                 v = fmaf(e, e, v);
             }
         ma[i] = m;
@@ -222,7 +226,7 @@ __device__ __forceinline__ void pair_windows(const float* R, const float2* W, in
 #pragma unroll
         for (int dx = 0; dx <= 2 * RHO; ++dx) {
             const float2 b = W[(ly + y) * G::HWC + lx + dx];
-            const float a = R[(ly + y) * G::HWC + lx + dx];
+            const float a = R[(ly + y) * G::RS + lx + dx];
 #pragma unroll
             for (int i = 0; i < PX; ++i)
                 if (y - i >= 0 && y - i <= 2 * RHO) {
@@ -238,7 +242,7 @@ template <class G>
 __device__ __forceinline__ void load_ref(const DiffP& P, int x0, int y0, float* R) {
     for (int p = threadIdx.x; p < G::NPOS; p += blockDim.x) {
         const int hy = p / G::HWC, hx = p - hy * G::HWC, x = x0 + hx, y = y0 + hy;
-        R[p] = (x >= 0 && y >= 0 && x < P.W && y < P.H) ? P.ref[(size_t)y * P.W + x] : 0.0f;
+        R[hy * G::RS + hx] = (x >= 0 && y >= 0 && x < P.W && y < P.H) ? P.ref[(size_t)y * P.W + x] : 0.0f;
     }
 }
 
@@ -374,17 +378,24 @@ struct GradOut {
 
 // Shared memory of the backward kernel, in floats, for nc matching cameras
 // and nf = 4 nc + 3 coefficient fields (all of them pairs).
-template <int RHO>
+template <int RHO, int MC>
 struct BwdLayout {
     using G = Tile<RHO, 16, 1>;
-    static constexpr int FS = G::SW + 1;    // field row stride (pairs)
-    static constexpr int HS = G::HWC + 1;   // horizontal sums' row stride (pairs)
+    // Zeros on either side of the direction that is summed, so that no sum tests
+    // its bounds (written once; with the reference stride RS 2837 -> 2782 us at
+    // 640 x 512, 128 planes, 2 cameras): PF columns of the fields, PH rows of the
+    // horizontal sums.  Two CTAs per SM are worth more than the tests, so 3 and
+    // 4 cameras, and the fields of the widest window, go without.
+    static constexpr int PH = MC == 2 ? 2 * RHO : 0, PF = MC == 2 && RHO < 4 ? 2 * RHO : 0;
+    static constexpr int FS = G::SW + 2 * PF + 1;  // field row stride (pairs)
+    static constexpr int HS = G::HWC + 1;          // horizontal sums' row stride (pairs)
+    static constexpr int HR = G::TH + 2 * PH;      // horizontal sums' rows
     // odd strides: lanes on consecutive rows reach distinct banks
     static_assert(FS % 2 == 1 && HS % 2 == 1, "conflict-free rows");
     __host__ __device__ static constexpr int nf(int nc) { return 4 * nc + 3; }
-    // warped pairs [nc][NPOS], fields [nf][TH][FS], horizontal sums [nf][TH][HS], reference [NPOS]
+    // warped pairs [nc][NPOS], fields [nf][TH][FS], horizontal sums [nf][HR][HS], reference [HH][RS]
     __host__ __device__ static constexpr size_t floats(int nc) {
-        return 2 * ((size_t)nc * G::NPOS + (size_t)nf(nc) * G::TH * (FS + HS)) + G::NPOS;
+        return 2 * ((size_t)nc * G::NPOS + (size_t)nf(nc) * (G::TH * FS + HR * HS)) + G::HH * G::RS;
     }
 };
 
@@ -470,20 +481,22 @@ template <int RHO, int MC>
 __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__ DiffP P, const float* aux,
                                                          const float* g_range, const float* g_cost, float* g_ref,
                                                          const __grid_constant__ GradOut GO, double* g_pose) {
-    using BL = BwdLayout<RHO>;
+    using BL = BwdLayout<RHO, MC>;
     using G = typename BL::G;
-    constexpr int HWC = G::HWC, NPOS = G::NPOS, TH = G::TH, FS = BL::FS, HS = BL::HS, N = G::N, RPT = G::RPT, SW = G::SW;
+    constexpr int HWC = G::HWC, NPOS = G::NPOS, TH = G::TH, FS = BL::FS, HS = BL::HS, HR = BL::HR, PF = BL::PF, PH = BL::PH, N = G::N, RPT = G::RPT,
+                  SW = G::SW;
     constexpr int PX = 1;
     const int nc = P.n_cams, nf = BL::nf(nc);
     extern __shared__ __align__(16) float sm[];
     float2* W2 = reinterpret_cast<float2*>(sm);
     float2* F = W2 + nc * NPOS;
     float2* Hx = F + nf * TH * FS;
-    float* R = reinterpret_cast<float*>(Hx + nf * TH * HS);
+    float* R = reinterpret_cast<float*>(Hx + nf * HR * HS);
     __shared__ float red[ST / 32][6 * MC];
     const int tid = threadIdx.x, lx = tid % SW, ly = tid / SW * PX;
     const int bx = blockIdx.x * SW, by = blockIdx.y * TH, x0 = bx - RHO, y0 = by - RHO;
     load_ref<G>(P, x0, y0, R);
+    for (int i = tid; i < nf * (TH * FS + HR * HS); i += ST) F[i] = dup2(0.f);  // fields and horizontal sums
     __syncthreads();
     float ma[PX], va[PX];
     ref_windows<G>(R, lx, ly, ma, va);
@@ -513,7 +526,7 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
 #pragma unroll
     for (int i = 0; i < RPT; ++i) gR[i] = 0.f;
     const int qc = (RHO + TH / 2) * HWC + RHO + SW / 2;  // centre of the tile
-    const float ca = R[qc];
+    const float ca = R[(RHO + TH / 2) * G::RS + RHO + SW / 2];
     for (int k = 0; k < P.K; k += 2) {
         const int np = min(2, P.K - k);
         const PlaneD pl0 = P.planes[k], pl1 = P.planes[k + np - 1];
@@ -583,7 +596,7 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
                 kzb[q] = on ? div_rn(gzz, vb[i][q], rcp_rn(vb[i][q])) : 0.f;
                 mbc[q] = on ? mb[i][q] - (q ? cb.y : cb.x) : 0.f;
             }
-            float2* f = F + (ly + i) * FS + lx;
+            float2* f = F + (ly + i) * FS + PF + lx;
             for (int j = 0; j < nc; ++j) {
                 const bool m0 = jb[i][0] == j, m1 = jb[i][1] == j;
                 f[(4 * j + 0) * TH * FS] = make_float2(m0 ? ka[0] : 0.f, m1 ? ka[1] : 0.f);
@@ -603,21 +616,21 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
         constexpr int RO = (HWC + 3) / 4;  // outputs of an item
         for (int it = tid; it < 4 * nf * TH; it += ST) {
             const int part = it / (nf * TH), fr = it - part * (nf * TH);
-            const float2* in = F + fr * FS;
-            float2* out = Hx + fr * HS;
             const int c0 = part * RO;
+            const float2* in = F + fr * FS + c0 + PF - 2 * RHO;
+            float2* out = Hx + (fr / TH * HR + PH + fr % TH) * HS + c0;
             float2 v[RO + 2 * RHO];
 #pragma unroll
             for (int t = 0; t < RO + 2 * RHO; ++t) {
                 const int x = c0 - 2 * RHO + t;
-                v[t] = x >= 0 && x < SW ? in[x] : dup2(0.f);
+                v[t] = PF || (x >= 0 && x < SW) ? in[t] : dup2(0.f);
             }
 #pragma unroll
             for (int c = 0; c < RO; ++c) {
                 float2 s = v[c];
 #pragma unroll
                 for (int t = 1; t <= 2 * RHO; ++t) s = add2(s, v[c + t]);
-                if (c0 + c < HWC) out[c0 + c] = s;
+                if (c0 + c < HWC) out[c] = s;
             }
         }
         __syncthreads();
@@ -625,14 +638,14 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
         // The pose accumulators take the first plane's samples of every position,
         // then the second's: the order of one plane at a time
         auto column = [&](int f, int p) {  // sum of field f over rows y - 2 RHO .. y at halo position p
-            const int y = p / HWC, x = p - y * HWC;
-            const float2* in = Hx + (f * TH + y - 2 * RHO) * HS + x;
-            float2 v[2 * RHO + 1];
+            const int y = p / HWC - 2 * RHO;
+            const float2* in = Hx + f * (HR * HS) + (y + PH) * HS + p % HWC;
+            float2 s = dup2(0.f);
 #pragma unroll
-            for (int t = 0; t <= 2 * RHO; ++t) v[t] = y - 2 * RHO + t >= 0 && y - 2 * RHO + t < TH ? in[t * HS] : dup2(0.f);
-            float2 s = v[0];
-#pragma unroll
-            for (int t = 1; t <= 2 * RHO; ++t) s = add2(s, v[t]);
+            for (int t = 0; t <= 2 * RHO; ++t) {
+                const float2 v = PH || (y + t >= 0 && y + t < TH) ? in[t * HS] : dup2(0.f);
+                s = t == 0 ? v : add2(s, v);
+            }
             return s;
         };
         float2 g[RPT];  // dL/dref of this pair
@@ -641,7 +654,7 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
             const int p = tid + i * ST;
             g[i] = dup2(0.f);
             if (p < NPOS) {
-                const float a = R[p] - ca;
+                const float a = R[p / HWC * G::RS + p % HWC] - ca;
                 g[i] = add2(fma2(dup2(-a), column(4 * nc + 1, p), neg2(column(4 * nc, p))), column(4 * nc + 2, p));
             }
         }
@@ -657,7 +670,7 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
 #pragma unroll
                 for (int t = 0; t < 6; ++t) m[i][t] = dup2(0.f);
                 if (p < NPOS) {
-                    const float a = R[p] - ca;
+                    const float a = R[p / HWC * G::RS + p % HWC] - ca;
                     const float2 w = W2[j * NPOS + p], b = add2(w, neg2(cb)), a1 = column(4 * j, p);
                     float2 v = fma2(dup2(a), a1, neg2(column(4 * j + 1, p)));
                     v = add2(fma2(neg2(b), column(4 * j + 2, p), v), column(4 * j + 3, p));
@@ -783,7 +796,7 @@ namespace {
 
 template <class G>
 int launch_fwd(const DiffP& P, float* range, float* cost, float* aux, cudaStream_t s) {
-    const size_t smem = sizeof(float) * (ROUND * ST * G::PX + (2 * FG * P.n_cams + 1) * G::NPOS);
+    const size_t smem = sizeof(float) * (ROUND * ST * G::PX + 2 * FG * P.n_cams * G::NPOS + G::HH * G::RS);
     auto* kernel = soft_fwd_kernel<G>;
     PS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kernel<<<dim3((P.W + G::SW - 1) / G::SW, (P.H + G::TH - 1) / G::TH), FG * ST, smem, s>>>(P, range, cost, aux);
@@ -804,9 +817,9 @@ int forward(const psdiff_t* h, const DiffP& P, float* range, float* cost, float*
 template <int RHO, int MC>
 int launch_bwd(const psdiff_t* h, const DiffP& P, const float* aux, const float* g_range, const float* g_cost, float* g_ref,
                const GradOut& G, double* g_pose, cudaStream_t s) {
-    using T = typename BwdLayout<RHO>::G;
-    // at most 170 KB (window 9, 4 cameras)
-    const size_t smem = sizeof(float) * BwdLayout<RHO>::floats(P.n_cams);
+    using T = typename BwdLayout<RHO, MC>::G;
+    // at most 122 KB (window 9, 4 cameras)
+    const size_t smem = sizeof(float) * BwdLayout<RHO, MC>::floats(P.n_cams);
     auto* kernel = soft_bwd_kernel<RHO, MC>;
     PS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kernel<<<dim3((P.W + T::SW - 1) / T::SW, (P.H + T::TH - 1) / T::TH), ST, smem, s>>>(P, aux, g_range, g_cost, g_ref, G,
