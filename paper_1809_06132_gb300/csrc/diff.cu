@@ -25,8 +25,8 @@
 //                    ref_to_cam pose (CTA reduction, FP64 atomics).
 // Both are bound by instruction issue and latency (DRAM holds the images and
 // ray table once).  A forward and backward pass through autograd, 640 x 512,
-// 128 planes, 2 cameras: 5.89 -> 4.09 ms (device time of the backward kernel
-// 4.22 -> 2.78 ms); 96 x 80, 32 planes: 672 -> 523 us.
+// 128 planes, 2 cameras: 5.89 -> 3.91 ms (device time of the backward kernel
+// 4.22 -> 2.57 ms); 96 x 80, 32 planes: 672 -> 523 us.
 // Before: one pixel per thread, general divisions and square roots (their
 // slow-path branches serialise a thread's samples), the reference window's
 // sums repeated per plane, and a backward of one plane at a time with seven
@@ -387,11 +387,17 @@ struct BwdLayout {
     // horizontal sums.  Two CTAs per SM are worth more than the tests, so 3 and
     // 4 cameras, and the fields of the widest window, go without.
     static constexpr int PH = MC == 2 ? 2 * RHO : 0, PF = MC == 2 && RHO < 4 ? 2 * RHO : 0;
-    static constexpr int FS = G::SW + 2 * PF + 1;  // field row stride (pairs)
-    static constexpr int HS = G::HWC + 1;          // horizontal sums' row stride (pairs)
-    static constexpr int HR = G::TH + 2 * PH;      // horizontal sums' rows
-    // odd strides: lanes on consecutive rows reach distinct banks
-    static_assert(FS % 2 == 1 && HS % 2 == 1, "conflict-free rows");
+    static constexpr int HR = G::TH + 2 * PH;        // horizontal sums' rows
+    static constexpr int RO = (G::HWC + 3) / 4;      // outputs of a horizontal item
+    // Row strides in pairs (16 of them span the banks).  HS = HWC: consecutive
+    // halo positions are consecutive words, so the vertical sums, most of the
+    // traffic, have no conflict and need no row index.  A half-warp of the
+    // horizontal sums takes 4 parts of 4 rows: with 5 outputs a part and strides
+    // of 4 or 12 mod 16 (windows 3 and 5; HS of window 5) all 16 words differ.
+    // Odd strides and a warp per part before: 2780 -> 2567 us (as above).
+    static constexpr int HS = G::HWC;
+    static constexpr int FS = RO != 5 ? G::SW + 2 * PF + 1 : PF ? 28 : 20;
+    static_assert(FS >= G::SW + 2 * PF && 4 * RO >= G::HWC, "rows hold their margins");
     __host__ __device__ static constexpr int nf(int nc) { return 4 * nc + 3; }
     // warped pairs [nc][NPOS], fields [nf][TH][FS], horizontal sums [nf][HR][HS], reference [HH][RS]
     __host__ __device__ static constexpr size_t floats(int nc) {
@@ -483,8 +489,8 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
                                                          const __grid_constant__ GradOut GO, double* g_pose) {
     using BL = BwdLayout<RHO, MC>;
     using G = typename BL::G;
-    constexpr int HWC = G::HWC, NPOS = G::NPOS, TH = G::TH, FS = BL::FS, HS = BL::HS, HR = BL::HR, PF = BL::PF, PH = BL::PH, N = G::N, RPT = G::RPT,
-                  SW = G::SW;
+    constexpr int HWC = G::HWC, NPOS = G::NPOS, TH = G::TH, SW = G::SW, FS = BL::FS, HS = BL::HS, HR = BL::HR, RO = BL::RO, PF = BL::PF,
+                  PH = BL::PH, N = G::N, RPT = G::RPT;
     constexpr int PX = 1;
     const int nc = P.n_cams, nf = BL::nf(nc);
     extern __shared__ __align__(16) float sm[];
@@ -613,10 +619,8 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
         // the row.  Direct sums, not running ones: coefficients of low-texture
         // windows are large, and a running sum would leave their rounding residue
         // where the exact sum is zero
-        constexpr int RO = (HWC + 3) / 4;  // outputs of an item
         for (int it = tid; it < 4 * nf * TH; it += ST) {
-            const int part = it / (nf * TH), fr = it - part * (nf * TH);
-            const int c0 = part * RO;
+            const int fr = it / 4, c0 = it % 4 * RO;
             const float2* in = F + fr * FS + c0 + PF - 2 * RHO;
             float2* out = Hx + (fr / TH * HR + PH + fr % TH) * HS + c0;
             float2 v[RO + 2 * RHO];
@@ -639,7 +643,7 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
         // then the second's: the order of one plane at a time
         auto column = [&](int f, int p) {  // sum of field f over rows y - 2 RHO .. y at halo position p
             const int y = p / HWC - 2 * RHO;
-            const float2* in = Hx + f * (HR * HS) + (y + PH) * HS + p % HWC;
+            const float2* in = Hx + f * (HR * HS) + (PH - 2 * RHO) * HS + p;
             float2 s = dup2(0.f);
 #pragma unroll
             for (int t = 0; t <= 2 * RHO; ++t) {
