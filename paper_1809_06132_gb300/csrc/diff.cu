@@ -393,7 +393,7 @@ struct BwdLayout {
     // halo positions are consecutive words, so the vertical sums, most of the
     // traffic, have no conflict and need no row index.  A half-warp of the
     // horizontal sums takes 4 parts of 4 rows: with 5 outputs a part and strides
-    // of 4 or 12 mod 16 (windows 3 and 5; HS of window 5) all 16 words differ.
+    // of 4 or 12 mod 16 (window 5) all 16 words differ.
     // Odd strides and a warp per part before: 2780 -> 2567 us (as above).
     static constexpr int HS = G::HWC;
     static constexpr int FS = RO != 5 ? G::SW + 2 * PF + 1 : PF ? 28 : 20;
