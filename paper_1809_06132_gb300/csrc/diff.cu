@@ -25,8 +25,8 @@
 //                    ref_to_cam pose (CTA reduction, FP64 atomics).
 // Both are bound by instruction issue and latency (DRAM holds the images and
 // ray table once).  A forward and backward pass through autograd, 640 x 512,
-// 128 planes, 2 cameras: 5.89 -> 3.91 ms (device time of the backward kernel
-// 4.22 -> 2.57 ms); 96 x 80, 32 planes: 672 -> 523 us.
+// 128 planes, 2 cameras: 5.93 -> 3.87 ms (device time of the backward kernel
+// 4.22 -> 2.57 ms); 96 x 80, 32 planes: 686 -> 537 us.
 // Before: one pixel per thread, general divisions and square roots (their
 // slow-path branches serialise a thread's samples), the reference window's
 // sums repeated per plane, and a backward of one plane at a time with seven

@@ -1,5 +1,5 @@
 """Soft sweep at the edges of its tiling (32 x 16 and 16 x 16 output tiles,
-plane pairs, rounds of 16 planes shared by 1 .. 8 CTAs): forward maps and
+plane pairs, rounds of 16 planes shared by two groups of threads): forward maps and
 gradients against the FP64 oracle, within the bounds the other soft-sweep
 tests use."""
 import numpy as np
