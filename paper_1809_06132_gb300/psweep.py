@@ -235,9 +235,20 @@ def _cuda_device(device, name: str):
 
 
 def _dev(t: torch.Tensor, dtype, name: str) -> int:
+    """Address of a tensor that the caller holds until the call that reads it
+    is launched: of a copy passed on directly nothing would be left, and the
+    next one made could take its place."""
     if not (t.is_cuda and t.dtype == dtype and t.is_contiguous()):
         raise ValueError(f"{name} must be a contiguous CUDA {dtype} tensor")
     return t.data_ptr()
+
+
+def _dense(t: torch.Tensor, stream) -> torch.Tensor:
+    """t, or a contiguous copy of it made on the stream of the call that reads it."""
+    if t.is_contiguous() or stream is None:
+        return t.contiguous()
+    with torch.cuda.stream(stream):
+        return t.contiguous()
 
 
 def level_shape(ref, lv):
@@ -637,9 +648,9 @@ class Tsdf:
     def load_blocks(self, keys: torch.Tensor, D: torch.Tensor, W: torch.Tensor, stream=None):
         """Insert or overwrite blocks (checkpoint resume, swap-in)."""
         n = keys.shape[0]
-        _check(load().tsdf_load(self.h, _dev(keys.contiguous(), torch.int32, "keys"),
-                                _dev(D.contiguous(), torch.float32, "D"), _dev(W.contiguous(), torch.float32, "W"),
-                                n, _stream_ptr(stream)))
+        keys, D, W = (_dense(t, stream) for t in (keys, D, W))
+        _check(load().tsdf_load(self.h, _dev(keys, torch.int32, "keys"), _dev(D, torch.float32, "D"),
+                                _dev(W, torch.float32, "W"), n, _stream_ptr(stream)))
 
     def extract(self, min_weight: float = 0.0, device="cuda", stream=None):
         """(keys (n, 3) int32, D (n, 512), W (n, 512)) as CUDA tensors, in pool order."""
@@ -795,8 +806,10 @@ class SoftSweep:
             gi = [torch.zeros_like(im) for im in images]
         gptr = (C.c_void_p * len(gi))(*[g.data_ptr() for g in gi])
         gp = torch.zeros((len(self.rig.cams), 6), dtype=torch.float64, device=images[0].device)
-        gr = _dev(g_range.contiguous(), torch.float32, "g_range") if g_range is not None else None
-        gc = _dev(g_cost.contiguous(), torch.float32, "g_cost") if g_cost is not None else None
+        g_range = _dense(g_range, stream) if g_range is not None else None
+        g_cost = _dense(g_cost, stream) if g_cost is not None else None
+        gr = _dev(g_range, torch.float32, "g_range") if g_range is not None else None
+        gc = _dev(g_cost, torch.float32, "g_cost") if g_cost is not None else None
         _check(load().psdiff_backward(self.h, ims, ps, _dev(aux, torch.float32, "aux"), gr, gc, gptr,
                                       gp.data_ptr(), _stream_ptr(stream)))
         return gi, gp
@@ -835,7 +848,8 @@ def soft_depth(sweep: SoftSweep, images, delta: Optional[torch.Tensor] = None, b
 def tsdf_dense_fuse_backward(voxels_in, dims, origin, voxel_size, mu, w_max, depth, cam, world_to_cam, g_D_out,
                              want_depth: bool = True, want_pose: bool = True, stream=None):
     """(dL/dD_in per voxel, dL/ddepth, (6,) float64 pose gradient) of one fusion step."""
-    gD = _dev(g_D_out.contiguous(), torch.float32, "g_D_out")
+    g_D_out = _dense(g_D_out, stream)
+    gD = _dev(g_D_out, torch.float32, "g_D_out")
     gin = torch.empty(g_D_out.shape, dtype=torch.float32, device=voxels_in.device)
     gd = torch.zeros(depth.shape, dtype=torch.float32, device=depth.device) if want_depth else None
     gp = torch.zeros(6, dtype=torch.float64, device=depth.device) if want_pose else None
