@@ -198,9 +198,13 @@ def camera(c) -> ps_camera:
 
 def pose(p) -> ps_pose:
     # one copy of the struct's 12 doubles: filling it element by element took 8 us a pose
+    R = np.asarray(p.R, dtype=np.float64).reshape(-1)
+    t = np.asarray(p.t, dtype=np.float64).reshape(-1)
+    if R.size < 9 or t.size < 3:   # (one value alone would be broadcast)
+        raise IndexError(f"a pose needs 9 values of R and 3 of t, got {R.size} and {t.size}")
     a = np.empty(12)
-    a[:9] = np.asarray(p.R, dtype=np.float64).reshape(-1)[:9]
-    a[9:] = np.asarray(p.t, dtype=np.float64).reshape(-1)[:3]
+    a[:9] = R[:9]
+    a[9:] = t[:3]
     return ps_pose.from_buffer_copy(a)
 
 
