@@ -225,8 +225,10 @@ def level(lv) -> ps_level:
 def boxes_array(boxes):
     b = np.zeros((0, 4), dtype=np.int32) if boxes is None else np.ascontiguousarray(boxes, dtype=np.int32)
     n = len(b)
-    if n and (b.ndim != 2 or b.shape[1] != 4):
-        raise ValueError(f"boxes must be (n, 4) integers, got {b.shape}")
+    if n and (b.ndim != 2 or b.shape[1] > 4):
+        raise TypeError(f"boxes must be (n, 4) integers, got {b.shape}")
+    if n and b.shape[1] < 4:   # what is left out is zero, as in a ps_box
+        b = np.ascontiguousarray(np.pad(b, ((0, 0), (0, 4 - b.shape[1]))))
     return ((ps_box * n).from_buffer_copy(b) if n else (ps_box * 1)()), n
 
 
