@@ -805,11 +805,10 @@ class SoftSweep:
     def backward(self, images, poses, aux, g_range=None, g_cost=None, stream=None):
         """(per-image gradients, (n_cams, 6) float64 pose gradients (w, v))."""
         ims, ps = self._args(images, poses)
-        if all(im.shape == images[0].shape for im in images):   # one buffer, cleared in one launch
-            gi = list(torch.zeros((len(images),) + tuple(images[0].shape), dtype=torch.float32,
-                                  device=images[0].device).unbind(0))
-        else:
-            gi = [torch.zeros_like(im) for im in images]
+        # a tensor of its own per image (slices of one would share its memory and
+        # version, and refuse some in-place operations), cleared in one launch
+        gi = [torch.empty_like(im) for im in images]
+        torch._foreach_zero_(gi)
         gptr = (C.c_void_p * len(gi))(*[g.data_ptr() for g in gi])
         gp = torch.zeros((len(self.rig.cams), 6), dtype=torch.float64, device=images[0].device)
         g_range = _dense(g_range, stream) if g_range is not None else None
