@@ -585,7 +585,9 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
 #pragma unroll
         for (int i = 0; i < PX; ++i) {
             const float4 ray = P.rays[use[i] ? (size_t)(by + ly + i) * P.W + bx + lx : 0];
-            float ka[2], kza[2], kzb[2], mac = ma[i] - ca, mbc[2];
+            // all of them zero where no camera wins: a window that holds a sample
+            // that is no number must not pass it on to its neighbours' sums
+            float ka[2], kza[2], kzb[2], mac[2], mbc[2];
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const PlaneD& pl = q == 0 ? pl0 : pl1;
@@ -600,19 +602,20 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
                 ka[q] = on ? div_rn(gz, sab[i][q], rcp_rn(sab[i][q])) : 0.f;
                 kza[q] = on ? div_rn(gzz, va[i], rcp_rn(va[i])) : 0.f;
                 kzb[q] = on ? div_rn(gzz, vb[i][q], rcp_rn(vb[i][q])) : 0.f;
+                mac[q] = on ? ma[i] - ca : 0.f;
                 mbc[q] = on ? mb[i][q] - (q ? cb.y : cb.x) : 0.f;
             }
             float2* f = F + (ly + i) * FS + PF + lx;
             for (int j = 0; j < nc; ++j) {
                 const bool m0 = jb[i][0] == j, m1 = jb[i][1] == j;
                 f[(4 * j + 0) * TH * FS] = make_float2(m0 ? ka[0] : 0.f, m1 ? ka[1] : 0.f);
-                f[(4 * j + 1) * TH * FS] = make_float2(m0 ? ka[0] * mac : 0.f, m1 ? ka[1] * mac : 0.f);
+                f[(4 * j + 1) * TH * FS] = make_float2(m0 ? ka[0] * mac[0] : 0.f, m1 ? ka[1] * mac[1] : 0.f);
                 f[(4 * j + 2) * TH * FS] = make_float2(m0 ? kzb[0] : 0.f, m1 ? kzb[1] : 0.f);
                 f[(4 * j + 3) * TH * FS] = make_float2(m0 ? kzb[0] * mbc[0] : 0.f, m1 ? kzb[1] * mbc[1] : 0.f);
             }
             f[(4 * nc + 0) * TH * FS] = make_float2(ka[0] * mbc[0], ka[1] * mbc[1]);
             f[(4 * nc + 1) * TH * FS] = make_float2(kza[0], kza[1]);
-            f[(4 * nc + 2) * TH * FS] = make_float2(kza[0] * mac, kza[1] * mac);
+            f[(4 * nc + 2) * TH * FS] = make_float2(kza[0] * mac[0], kza[1] * mac[1]);
         }
         __syncthreads();
         // 3a. horizontal box sums: halo column c collects pixels c - 2 RHO .. c of
