@@ -40,6 +40,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "sweep_dev.cuh"
@@ -55,6 +56,7 @@ struct DiffCam {
     float r2_max;
     // projection constants, and those of its derivative, as (value, value) pairs
     float2 R2[9], t2[3], xi, fx, fy, cx, cy, k1, k2, k2x2, p1, p1x2, p1x6, p2, p2x2, p2x6, lim;
+    float u_max, v_max;  // largest coordinates inside the image (read for wide images)
 };
 
 struct DiffP {
@@ -116,16 +118,23 @@ __device__ __forceinline__ Proj project_pair(const DiffCam& C, const PlaneD& p0,
 
 // The bilinear cell of camera C at (u, v), clamped into the image: corner
 // offsets and weights; false when (u, v) lies outside [0, W-1] x [0, H-1].
+// WIDE: images of 2^31 texels or more, or of a side above 2^24, whose offsets
+// take 64 bits and whose last coordinate may be no float (64 bits for every
+// image: 640 x 512, 128 planes, 2 cameras 1250 -> 1280 us forward, 2475 ->
+// 2518 backward; an index per row more still).
+template <bool WIDE>
 struct Cell {
-    int i00, i10, i01, i11;
+    std::conditional_t<WIDE, long long, int> i00, i10, i01, i11;
     float ax, ay;
 };
-__device__ __forceinline__ bool cell_at(const DiffCam& C, float u, float v, Cell& c) {
-    const float uc = fminf(fmaxf(u, 0.0f), (float)(C.width - 1)), vc = fminf(fmaxf(v, 0.0f), (float)(C.height - 1));
+template <bool WIDE>
+__device__ __forceinline__ bool cell_at(const DiffCam& C, float u, float v, Cell<WIDE>& c) {
+    const float uc = fminf(fmaxf(u, 0.0f), WIDE ? C.u_max : (float)(C.width - 1)),
+                vc = fminf(fmaxf(v, 0.0f), WIDE ? C.v_max : (float)(C.height - 1));
     int x = (int)uc, y = (int)vc;
     if (!PS_DCHECK(x >= 0 && y >= 0 && x < C.width && y < C.height, CHK_GATHER)) x = y = 0;
     const int dx = x < C.width - 1 ? 1 : 0, dy = y < C.height - 1 ? C.width : 0;
-    c.i00 = y * C.width + x;
+    c.i00 = static_cast<decltype(c.i00)>(y) * C.width + x;
     c.i10 = c.i00 + dx;
     c.i01 = c.i00 + dy;
     c.i11 = c.i01 + dx;
@@ -138,10 +147,11 @@ __device__ __forceinline__ bool cell_at(const DiffCam& C, float u, float v, Cell
 // y: p1); NaN where invalid (no ray, plane behind the ray, no projection,
 // outside the image).  The gathers are clamped into the image and always
 // issued, so nothing branches and a thread's positions overlap.
+template <bool WIDE>
 __device__ __forceinline__ float2 warp_pair(const DiffCam& C, const PlaneD& p0, const PlaneD& p1, const float4& r) {
     const float nan = __int_as_float(0x7fc00000);
     const Proj o = project_pair(C, p0, p1, r);
-    Cell a, b;
+    Cell<WIDE> a, b;
     const bool in0 = cell_at(C, o.u.x, o.v.x, a), in1 = cell_at(C, o.u.y, o.v.y, b);
     const float* I = C.img;
     const float w0 = bilerp(a.ax, a.ay, I[a.i00], I[a.i10], I[a.i01], I[a.i11]);
@@ -253,14 +263,14 @@ __device__ __forceinline__ float4 ray_at(const DiffP& P, int x, int y) {
 }
 
 // Warped sample pairs of the halo, every camera, by the ST threads tid.
-template <class G>
+template <class G, bool WIDE>
 __device__ __forceinline__ void warp_tile(const DiffP& P, const PlaneD& pl0, const PlaneD& pl1, int x0, int y0, int tid,
                                           float2* W2) {
     for (int j = 0; j < P.n_cams; ++j)
 #pragma unroll
         for (int i = 0; i < G::RPT; ++i) {
             const int p = tid + i * ST;
-            if (p < G::NPOS) W2[j * G::NPOS + p] = warp_pair(P.cams[j], pl0, pl1, ray_at(P, x0 + p % G::HWC, y0 + p / G::HWC));
+            if (p < G::NPOS) W2[j * G::NPOS + p] = warp_pair<WIDE>(P.cams[j], pl0, pl1, ray_at(P, x0 + p % G::HWC, y0 + p / G::HWC));
         }
 }
 
@@ -274,7 +284,7 @@ __device__ __forceinline__ void warp_tile(const DiffP& P, const PlaneD& pl0, con
 constexpr int FG = 2;
 constexpr int ROUND = 16;
 
-template <class G>
+template <class G, bool WIDE>
 __global__ void __launch_bounds__(FG * ST, 1) soft_fwd_kernel(const __grid_constant__ DiffP P, float* range, float* cost,
                                                               float* aux) {
     constexpr int RHO = G::RHO, PX = G::PX, SW = G::SW, NPIX = ST * PX;
@@ -305,7 +315,7 @@ __global__ void __launch_bounds__(FG * ST, 1) soft_fwd_kernel(const __grid_const
             const int k = k0 + 2 * group, np = max(0, min(2, n - k));
             const PlaneD pl0 = P.planes[base + min(k, n - 1)], pl1 = P.planes[base + min(k + 1, n - 1)];
             __syncthreads();  // the previous pairs' windows are done
-            warp_tile<G>(P, pl0, pl1, bx - RHO, by - RHO, tid, W2);
+            warp_tile<G, WIDE>(P, pl0, pl1, bx - RHO, by - RHO, tid, W2);
             __syncthreads();
             float2 best[PX];
 #pragma unroll
@@ -413,10 +423,11 @@ struct BwdLayout {
 // The warp is the forward's; g comes from reverse-mode differentiation of the
 // projection: the adjoints of the distorted point, of the normalised point
 // (mx, my), then of X through mx = X / den, my = Y / den, den = xi |X| + Z.
+template <bool WIDE>
 __device__ __forceinline__ void chain_pair(const DiffCam& C, const PlaneD& p0, const PlaneD& p1, const float4& r,
                                            float2 gw, float* img, float2 (&m)[6]) {
     const Proj o = project_pair(C, p0, p1, r);
-    Cell c[2];
+    Cell<WIDE> c[2];
     cell_at(C, o.u.x, o.v.x, c[0]);
     cell_at(C, o.u.y, o.v.y, c[1]);
     float2 gu, gv;
@@ -452,7 +463,7 @@ __device__ __forceinline__ void chain_pair(const DiffCam& C, const PlaneD& p0, c
         for (int q = 0; q < 2; ++q) {
             const float g = q ? gw.y : gw.x, ax = c[q].ax, ay = c[q].ay;
             if (g == 0.f) continue;
-            if (!PS_DCHECK(c[q].i00 >= 0 && c[q].i11 < C.width * C.height, CHK_GATHER)) continue;
+            if (!PS_DCHECK(c[q].i00 >= 0 && (long long)c[q].i11 < (long long)C.width * C.height, CHK_GATHER)) continue;
             atomicAdd(&img[c[q].i00], g * (1.f - ax) * (1.f - ay));
             atomicAdd(&img[c[q].i10], g * ax * (1.f - ay));
             atomicAdd(&img[c[q].i01], g * (1.f - ax) * ay);
@@ -483,7 +494,7 @@ __device__ __forceinline__ void chain_pair(const DiffCam& C, const PlaneD& p0, c
 // After the planes: dL/dref of the halo (global atomics) and the CTA's pose
 // gradient (FP64 atomics).  MC: most cameras (their pose accumulators are
 // registers).
-template <int RHO, int MC>
+template <int RHO, int MC, bool WIDE>
 __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__ DiffP P, const float* aux,
                                                          const float* g_range, const float* g_cost, float* g_ref,
                                                          const __grid_constant__ GradOut GO, double* g_pose) {
@@ -537,7 +548,7 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
         const int np = min(2, P.K - k);
         const PlaneD pl0 = P.planes[k], pl1 = P.planes[k + np - 1];
         __syncthreads();  // the previous pair's chain is done with the samples and sums
-        warp_tile<G>(P, pl0, pl1, x0, y0, tid, W2);
+        warp_tile<G, WIDE>(P, pl0, pl1, x0, y0, tid, W2);
         __syncthreads();
         // the per-camera centre of this pair's warped samples (a broadcast read)
         auto centre = [&](int j) {
@@ -692,7 +703,7 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
                         g[i].y = gb.y;
                     }
                     if (gw[i].x != 0.f || gw[i].y != 0.f)
-                        chain_pair(P.cams[j], pl0, pl1, ray_at(P, x0 + p % HWC, y0 + p / HWC), gw[i], GO.cam[j], m[i]);
+                        chain_pair<WIDE>(P.cams[j], pl0, pl1, ray_at(P, x0 + p % HWC, y0 + p / HWC), gw[i], GO.cam[j], m[i]);
                 }
             }
             // (a plane with gw = 0 may hold a sample that does not project)
@@ -762,6 +773,21 @@ void free_diff(psdiff_t* h) {
     delete h;
 }
 
+// Largest float not above n - 1.
+float last_coordinate(int n) {
+    const float x = (float)(n - 1);
+    return (double)x > (double)(n - 1) ? std::nextafter(x, 0.0f) : x;
+}
+
+// A matching image whose offsets do not fit 32 bits, or whose coordinates are not all floats.
+bool wide(const psdiff_t* h) {
+    for (int j = 0; j < h->n_cams; ++j) {
+        const ps_camera& c = h->cams[j];
+        if ((long long)c.width * c.height > INT32_MAX || c.width > 1 << 24 || c.height > 1 << 24) return true;
+    }
+    return false;
+}
+
 int fill_params(const psdiff_t* h, const float* const* images, const ps_pose* ref_to_cam, DiffP& P) {
     std::memset(&P, 0, sizeof(P));
     P.W = h->ref.width;
@@ -792,6 +818,8 @@ int fill_params(const psdiff_t* h, const float* const* images, const ps_pose* re
         D.r2_max = c.r2_max;
         D.width = c.width;
         D.height = c.height;
+        D.u_max = last_coordinate(c.width);
+        D.v_max = last_coordinate(c.height);
         D.img = images[1 + j];
     }
     return PS_OK;
@@ -801,10 +829,10 @@ int fill_params(const psdiff_t* h, const float* const* images, const ps_pose* re
 
 namespace {
 
-template <class G>
+template <class G, bool WIDE>
 int launch_fwd(const DiffP& P, float* range, float* cost, float* aux, cudaStream_t s) {
     const size_t smem = sizeof(float) * (ROUND * ST * G::PX + 2 * FG * P.n_cams * G::NPOS + G::HH * G::RS);
-    auto* kernel = soft_fwd_kernel<G>;
+    auto* kernel = soft_fwd_kernel<G, WIDE>;
     PS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kernel<<<dim3((P.W + G::SW - 1) / G::SW, (P.H + G::TH - 1) / G::TH), FG * ST, smem, s>>>(P, range, cost, aux);
     PS_CUDA(cudaGetLastError());
@@ -812,22 +840,24 @@ int launch_fwd(const DiffP& P, float* range, float* cost, float* aux, cudaStream
 }
 
 // Tiles of 32 x 16 pixels, two under each other per thread; images of too few
-// of them for the SMs take twice as many of 16 x 16.
+// of them for the SMs take twice as many of 16 x 16.  (Wide images, whose
+// time is their own size, have the small tiles and the four-camera layout.)
 template <int RHO>
 int forward(const psdiff_t* h, const DiffP& P, float* range, float* cost, float* aux, cudaStream_t s) {
     using Wide = Tile<RHO, 32, 2>;
     const long long tiles = (long long)((P.W + Wide::SW - 1) / Wide::SW) * ((P.H + Wide::TH - 1) / Wide::TH);
-    return tiles >= h->sms ? launch_fwd<Wide>(P, range, cost, aux, s)
-                           : launch_fwd<Tile<RHO, 16, 1>>(P, range, cost, aux, s);
+    if (wide(h)) return launch_fwd<Tile<RHO, 16, 1>, true>(P, range, cost, aux, s);
+    return tiles >= h->sms ? launch_fwd<Wide, false>(P, range, cost, aux, s)
+                           : launch_fwd<Tile<RHO, 16, 1>, false>(P, range, cost, aux, s);
 }
 
-template <int RHO, int MC>
+template <int RHO, int MC, bool WIDE>
 int launch_bwd(const psdiff_t* h, const DiffP& P, const float* aux, const float* g_range, const float* g_cost, float* g_ref,
                const GradOut& G, double* g_pose, cudaStream_t s) {
     using T = typename BwdLayout<RHO, MC>::G;
     // at most 122 KB (window 9, 4 cameras)
     const size_t smem = sizeof(float) * BwdLayout<RHO, MC>::floats(P.n_cams);
-    auto* kernel = soft_bwd_kernel<RHO, MC>;
+    auto* kernel = soft_bwd_kernel<RHO, MC, WIDE>;
     PS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kernel<<<dim3((P.W + T::SW - 1) / T::SW, (P.H + T::TH - 1) / T::TH), ST, smem, s>>>(P, aux, g_range, g_cost, g_ref, G,
                                                                                        g_pose);
@@ -928,8 +958,16 @@ extern "C" int psdiff_backward(psdiff_t* h, const float* const* images, const ps
     GradOut G;
     for (int j = 0; j < PS_MAX_CAMS; ++j) G.cam[j] = (g_images && j < h->n_cams) ? g_images[1 + j] : nullptr;
     cudaStream_t s = (cudaStream_t)stream;
-    auto go = h->n_cams <= 2 ? (P.rho == 2 ? launch_bwd<2, 2> : P.rho == 3 ? launch_bwd<3, 2> : launch_bwd<4, 2>)
-                             : (P.rho == 2 ? launch_bwd<2, 4> : P.rho == 3 ? launch_bwd<3, 4> : launch_bwd<4, 4>);
+    if (wide(h)) {
+        auto go = P.rho == 2 ? launch_bwd<2, 4, true> : P.rho == 3 ? launch_bwd<3, 4, true> : launch_bwd<4, 4, true>;
+        return go(h, P, aux, g_range, g_cost, g_ref, G, g_pose, s);
+    }
+    auto go = h->n_cams <= 2 ? (P.rho == 2   ? launch_bwd<2, 2, false>
+                                : P.rho == 3 ? launch_bwd<3, 2, false>
+                                             : launch_bwd<4, 2, false>)
+                             : (P.rho == 2   ? launch_bwd<2, 4, false>
+                                : P.rho == 3 ? launch_bwd<3, 4, false>
+                                             : launch_bwd<4, 4, false>);
     return go(h, P, aux, g_range, g_cost, g_ref, G, g_pose, s);
 }
 
