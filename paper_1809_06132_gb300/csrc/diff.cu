@@ -829,12 +829,15 @@ int fill_params(const psdiff_t* h, const float* const* images, const ps_pose* re
 
 namespace {
 
+// A kernel's shared-memory limit belongs to the process: every call sets the
+// same one, that of the most cameras, so that calls of several threads never
+// lower each other's between the attribute and the launch.
 template <class G, bool WIDE>
 int launch_fwd(const DiffP& P, float* range, float* cost, float* aux, cudaStream_t s) {
-    const size_t smem = sizeof(float) * (ROUND * ST * G::PX + 2 * FG * P.n_cams * G::NPOS + G::HH * G::RS);
+    auto smem = [](int nc) { return sizeof(float) * (ROUND * ST * G::PX + 2 * FG * nc * G::NPOS + G::HH * G::RS); };
     auto* kernel = soft_fwd_kernel<G, WIDE>;
-    PS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kernel<<<dim3((P.W + G::SW - 1) / G::SW, (P.H + G::TH - 1) / G::TH), FG * ST, smem, s>>>(P, range, cost, aux);
+    PS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(PS_MAX_CAMS)));
+    kernel<<<dim3((P.W + G::SW - 1) / G::SW, (P.H + G::TH - 1) / G::TH), FG * ST, smem(P.n_cams), s>>>(P, range, cost, aux);
     PS_CUDA(cudaGetLastError());
     return PS_OK;
 }
@@ -855,12 +858,12 @@ template <int RHO, int MC, bool WIDE>
 int launch_bwd(const psdiff_t* h, const DiffP& P, const float* aux, const float* g_range, const float* g_cost, float* g_ref,
                const GradOut& G, double* g_pose, cudaStream_t s) {
     using T = typename BwdLayout<RHO, MC>::G;
-    // at most 122 KB (window 9, 4 cameras)
-    const size_t smem = sizeof(float) * BwdLayout<RHO, MC>::floats(P.n_cams);
+    // at most 122 KB (window 9, 4 cameras); the limit as in launch_fwd
+    auto smem = [](int nc) { return sizeof(float) * BwdLayout<RHO, MC>::floats(nc); };
     auto* kernel = soft_bwd_kernel<RHO, MC, WIDE>;
-    PS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kernel<<<dim3((P.W + T::SW - 1) / T::SW, (P.H + T::TH - 1) / T::TH), ST, smem, s>>>(P, aux, g_range, g_cost, g_ref, G,
-                                                                                       g_pose);
+    PS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(MC)));
+    kernel<<<dim3((P.W + T::SW - 1) / T::SW, (P.H + T::TH - 1) / T::TH), ST, smem(P.n_cams), s>>>(P, aux, g_range, g_cost,
+                                                                                                 g_ref, G, g_pose);
     PS_CUDA(cudaGetLastError());
     return PS_OK;
 }
