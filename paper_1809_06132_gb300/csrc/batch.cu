@@ -228,7 +228,10 @@ extern "C" int psbatch_create(psweep_t* const* sweeps, int32_t n, const ps_batch
             PS_ARG(false, "psbatch_create: a work item needs %zu bytes of shared memory (device: %d)",
                    smem + fa.sharedSizeBytes, optin);
         }
-        PB_TRY(cudaFuncSetAttribute(b->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        // the kernel's limit belongs to the process: the device's own, which no
+        // other batch with this kernel lowers
+        PB_TRY(cudaFuncSetAttribute(b->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    optin - (int)fa.sharedSizeBytes));
         PB_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b->kernel, NT, smem));
         if (per_sm < 1) {
             free_batch(b);
