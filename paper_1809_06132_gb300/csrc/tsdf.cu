@@ -167,6 +167,14 @@ __device__ __forceinline__ bool slab(float A, float D, float inv, float lo, floa
     return t1 > t0;
 }
 
+// Index of the block that holds coordinate x (inv = 1 / block): x / block
+// rounded as a division, and infinite where that overflows (div_rn alone would
+// make it no number, which no bound of the local map cuts off).
+__device__ __forceinline__ float block_index(float x, float block, float inv) {
+    const float q = __fmul_rn(x, inv);
+    return floorf(fabsf(q) < __int_as_float(0x7f800000) ? div_rn(x, block, inv) : q);
+}
+
 // Blocks crossed by the segment [d - mu, d + mu] of every pixel's ray, and
 // the frame's largest range.  The candidates of a segment are cut axis by
 // axis, so that a row of blocks that it misses costs one test; the
@@ -199,8 +207,8 @@ __global__ void __launch_bounds__(128) alloc_kernel(const __grid_constant__ Fram
         const float Bp = fmaf(s1, dw[i], F.C[i]);
         Dv[i] = Bp - A[i];
         inv[i] = rcp_rn(Dv[i]);  // (not used where Dv is zero)
-        float flo = floorf(div_rn(fminf(A[i], Bp), F.block, F.inv_block));
-        float fhi = floorf(div_rn(fmaxf(A[i], Bp), F.block, F.inv_block));
+        float flo = block_index(fminf(A[i], Bp), F.block, F.inv_block);
+        float fhi = block_index(fmaxf(A[i], Bp), F.block, F.inv_block);
         if (F.gate) {
             // only blocks whose centre lies in the local map can be allocated:
             // clip the candidates to the gate's index range (one block of slack;

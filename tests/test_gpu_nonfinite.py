@@ -1,10 +1,13 @@
 """Values at the ends of FP32, and what they may and may not reach."""
 import dataclasses
 
+import numpy as np
 import pytest
 import torch
 
 import scenes
+from scenes.configs import TsdfParams
+from scenes.render import Pose
 
 pytestmark = pytest.mark.gpu
 
@@ -30,3 +33,24 @@ def test_a_reference_pixel_that_is_no_number(window):
     bad = ~torch.isfinite(gi[0])
     bad[y, x] = False        # (its own gradient has no value)
     assert not bad.any() and gi[0].nan_to_num().any()
+
+
+def _far_map(local_half):
+    cam = scenes.Camera(xi=1.0, fx=40.0, fy=40.0, cx=24.0, cy=20.0, width=48, height=40)
+    p = TsdfParams(voxel_size=0.02, mu=0.1, w_max=100.0, hash_slots=1 << 16, pool_blocks=1 << 14, local_half=local_half)
+    # the optical axis along (1, 1, 1): every coordinate of the far point overflows a block count
+    z = np.ones(3) / np.sqrt(3.0)
+    x = np.array([1.0, -1.0, 0.0]) / np.sqrt(2.0)
+    pose = Pose(np.stack([x, np.cross(z, x), z]), np.zeros(3))
+    depth = torch.zeros((40, 48), device="cuda")
+    depth[20, 24] = 2e38
+    return P.Tsdf(p, cam), depth, pose
+
+
+def test_a_range_beyond_the_largest_block_count():
+    m, depth, pose = _far_map((3.0, 3.0, 3.0))
+    m.integrate(depth, pose, (0.0, 0.0, 0.0))
+    assert m.status() == P.PS_OK and m.count() == 0    # outside the local map: skipped
+    m, depth, pose = _far_map(None)
+    m.integrate(depth, pose)
+    assert m.status() == P.PS_ERR_CAPACITY and m.count() == 0    # no local map: no key holds such a block
