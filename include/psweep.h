@@ -398,7 +398,8 @@ int tsdf_profile_read(tsdf_t* t, double* stage_ms, int32_t* n_calls);
  *   voxels        device float32: n_blocks x 512 {D, w} pairs; block
  *                 b = bx + nbx (by + nby bz) of the grid, voxel x + 8 y + 64 z
  *                 inside a block (the order tsdf_extract reports for a dense
- *                 map).  Zero it to start an empty map.
+ *                 map), aligned to 16 bytes (else PS_ERR_ARG).  Zero it to
+ *                 start an empty map.
  *   dims          host int32[3]: voxels per axis, multiples of 8, at most
  *                 PS_STATIC_MAX_BLOCKS blocks in all (larger grids get
  *                 PS_ERR_ARG and a message naming the limit).  The library
@@ -556,10 +557,10 @@ void psdiff_destroy(psdiff_t* h);
 
 /* Gradient of one fusion step into a caller-owned dense grid (the step
  * tsdf_integrate_dense_static performs; Eq. 2 with unit observation
- * weight): voxels_in is the grid BEFORE the step (same layout), g_D_out the
- * gradient with respect to the D of every voxel after it (float32 per
- * voxel; weights are counts and carry none).  Writes g_D_in (float32 per
- * voxel, may be NULL); ADDS to g_depth (device float32 H x W of cam, may be
+ * weight): voxels_in is the grid BEFORE the step (same layout; aligned to 8
+ * bytes, else PS_ERR_ARG), g_D_out the gradient with respect to the D of
+ * every voxel after it (float32 per voxel; weights are counts and carry
+ * none).  Writes g_D_in (float32 per voxel, may be NULL); ADDS to g_depth (device float32 H x W of cam, may be
  * NULL) and g_pose (device double[6], a left perturbation (w, v) of
  * world_to_cam, may be NULL).  An observed voxel (eta >= -mu) passes
  * w / (w + 1) of its gradient to D_in; if eta < mu also 1 / (mu (w + 1)) to
@@ -571,9 +572,9 @@ int tsdf_dense_fuse_backward(const float* voxels_in, const int32_t* dims, const 
                              double* g_pose, void* stream);
 
 /* The same gradient for a whole grid: g_out and g_in are {D, w} pairs like
- * voxels_in (8-byte aligned; the weights' part of g_out is not read, that of
- * g_in is written as zero), and g_depth and g_pose (either may be NULL) are
- * WRITTEN, not added to.  Asynchronous on `stream`; allocates nothing. */
+ * voxels_in (aligned to 8 bytes, else PS_ERR_ARG; the weights' part of g_out
+ * is not read, that of g_in is written as zero), and g_depth and g_pose
+ * (either may be NULL) are WRITTEN, not added to.  Asynchronous on `stream`; allocates nothing. */
 int tsdf_dense_fuse_backward_grid(const float* voxels_in, const int32_t* dims, const double* origin, double voxel_size,
                                   double mu, double w_max, const float* depth, const ps_camera* cam,
                                   const ps_pose* world_to_cam, const float* g_out, float* g_in, float* g_depth,

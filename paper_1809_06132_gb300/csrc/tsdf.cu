@@ -1065,6 +1065,9 @@ __global__ void static_dense_keys_kernel(int4* keys, int* n_alloc, int nx, int n
 namespace ps {
 namespace {
 
+// Vector accesses need their whole width's alignment, which no pointer type says.
+bool aligned(const void* p, uintptr_t bytes) { return reinterpret_cast<uintptr_t>(p) % bytes == 0; }
+
 // Frame record of a caller-owned dense grid at `origin` (no local map).
 int dense_frame(const double* origin, double voxel_size, double mu, double w_max, const ps_camera* cam,
                 const ps_pose* w2c, FrameP& F) {
@@ -1161,6 +1164,7 @@ extern "C" int tsdf_integrate_dense_static(float* voxels, const int32_t* dims, c
                                            const ps_camera* cam, const ps_pose* w2c, void* stream) {
     clear_error();
     PS_ARG(voxels && dims && origin && depth && cam && w2c, "tsdf_integrate_dense_static: NULL argument");
+    PS_ARG(aligned(voxels, 16), "tsdf_integrate_dense_static: voxels must be aligned to 16 bytes");
     PS_ARG(voxel_size > 0 && mu > 0 && w_max >= 1, "tsdf_integrate_dense_static: need voxel_size > 0, mu > 0, w_max >= 1");
     PS_ARG(cam->width > 0 && cam->height > 0 && cam->fx > 0 && cam->fy > 0 && cam->xi >= 0,
            "tsdf_integrate_dense_static: bad camera");
@@ -1218,6 +1222,9 @@ int dense_backward(const float* voxels_in, const int32_t* dims, const double* or
                    float* g_D_in, float* g_depth, double* g_pose, bool pairs, void* stream) {
     clear_error();
     PS_ARG(voxels_in && dims && origin && depth && cam && w2c && g_D_out, "tsdf_dense_fuse_backward: NULL argument");
+    PS_ARG(aligned(voxels_in, 8), "tsdf_dense_fuse_backward: voxels_in must be aligned to 8 bytes");
+    PS_ARG(!pairs || (aligned(g_D_out, 8) && aligned(g_D_in, 8)),
+           "tsdf_dense_fuse_backward_grid: g_out and g_in must be aligned to 8 bytes");
     PS_ARG(voxel_size > 0 && mu > 0 && w_max >= 1, "tsdf_dense_fuse_backward: need voxel_size > 0, mu > 0, w_max >= 1");
     PS_ARG(cam->width > 0 && cam->height > 0 && cam->fx > 0 && cam->fy > 0 && cam->xi >= 0,
            "tsdf_dense_fuse_backward: bad camera");

@@ -876,6 +876,8 @@ class _DenseFuseFn(torch.autograd.Function):
         d = delta.detach().cpu().double().numpy().reshape(6)
         p = se3_exp_left(d, base_pose)
         vin = vox_in.contiguous()
+        if vin.data_ptr() % 8:   # a view that starts between pairs
+            vin = vin.clone()
         dep = depth.contiguous()
         out = vin.clone()
         tsdf_integrate_dense_static(out, dims, origin, vs, mu, w_max, dep, cam, p)
