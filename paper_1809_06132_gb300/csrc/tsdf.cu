@@ -147,9 +147,9 @@ __device__ __forceinline__ bool pool_full(const TsdfDev& T) { return *((volatile
 
 // ----------------------------------------------------------------- kernels
 
-__global__ void depth_max_kernel(const float* depth, int n, unsigned* dmax_bits) {
+__global__ void depth_max_kernel(const float* depth, long long n, unsigned* dmax_bits) {
     float m = 0.f;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    for (long long i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         float d = depth[i];
         if (d > m && d < 3.0e38f) m = d;
     }
@@ -369,8 +369,8 @@ __device__ __forceinline__ void update_pair(const FrameP& F, const float* depth,
         const float pu = floorf((q ? u.y : u.x) + 0.5f), pv = floorf((q ? v.y : v.x) + 0.5f);
         const bool ok = (q ? Z.y > ln.y : Z.x > ln.x) && (q ? r2.y : r2.x) <= c.r2_max && pu >= 0.f && pv >= 0.f &&
                         pu < (float)c.width && pv < (float)c.height;
-        const int pix = ok ? (int)pv * c.width + (int)pu : 0;
-        if (!PS_DCHECK(pix >= 0 && pix < c.width * c.height, CHK_PIXEL)) continue;
+        const long long pix = ok ? (long long)(int)pv * c.width + (int)pu : 0;  // a map may hold more than 2^31
+        if (!PS_DCHECK(pix >= 0 && pix < (long long)c.width * c.height, CHK_PIXEL)) continue;
         const float d = ok ? __ldg(&depth[pix]) : 0.f;
         if (!(d > 0.f) || !(d < 3.0e38f)) continue;
         const float eta = voxel_eta(F, ax + q, ay, az, d);
@@ -799,7 +799,7 @@ extern "C" int tsdf_integrate(tsdf_t* t, const float* depth, const ps_pose* w2c,
     t->prof.mark(0, s);
     PS_CUDA(cudaMemsetAsync(t->T.n_vis, 0, 2 * sizeof(int), s));
     if (t->dense) {
-        depth_max_kernel<<<t->sms * 2, 256, 0, s>>>(depth, W * H, t->T.dmax_bits);
+        depth_max_kernel<<<t->sms * 2, 256, 0, s>>>(depth, (long long)W * H, t->T.dmax_bits);
         PS_CUDA(cudaGetLastError());
     }
     t->prof.mark(1, s);
@@ -1204,7 +1204,7 @@ extern "C" int tsdf_integrate_dense_static(float* voxels, const int32_t* dims, c
     static_dense_keys_kernel<<<(int)((n_blocks + 255) / 256), 256, 0, s>>>(T.pool_keys, T.n_alloc, (int)nx, (int)ny,
                                                                            (int)nz);
     PS_CUDA(cudaGetLastError());
-    depth_max_kernel<<<sms * 2, 256, 0, s>>>(depth, W * H, T.dmax_bits);
+    depth_max_kernel<<<sms * 2, 256, 0, s>>>(depth, (long long)W * H, T.dmax_bits);
     PS_CUDA(cudaGetLastError());
     visible_kernel<<<sms * 4, 256, 0, s>>>(F, T);
     PS_CUDA(cudaGetLastError());
