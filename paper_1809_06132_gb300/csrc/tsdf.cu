@@ -277,86 +277,34 @@ __global__ void visible_kernel(const __grid_constant__ FrameP F, TsdfDev T) {
     }
 }
 
-// Observation of a voxel by the depth map (Sec. III-C): eta, the pixel index
-// and the point in the camera frame.  a = voxel index - camera voxel (exact
-// int), F.fb the sub-voxel part, so the voxel centre sits at vox * (a + fb)
-// from the camera.  False when the voxel does not project into the image or
-// its pixel has no depth; eta < -mu is left to the caller.
-__device__ __forceinline__ bool observe_voxel(const FrameP& F, const float* depth, int ax, int ay, int az, float* eta_out,
-                                              size_t* pix_out, float Xc[3]) {
+// Two voxels seen by the depth map (Sec. III-C): (ax, ay, az) and its +x
+// neighbour, a = voxel index - camera voxel (exact int), F.fb the sub-voxel
+// part, so that a voxel's centre sits at vox * (a + fb) from the camera.  The
+// points in the camera frame, and for each the pixel and its depth, 0 where
+// the voxel does not project into the image or the pixel has no depth.
+// Forward and backward share this and voxel_eta, and every rounding in them
+// is written out: which voxels are observed, by which pixel and on which side
+// of -mu must not depend on the contractions that a compiler picks in each.
+// Packed pairs with branch-free quotients and roots: the general forms' slow
+// paths made the voxels of a thread wait for each other (ring-type maps of
+// 2 cm voxels were bound by that, not by HBM).
+struct Seen {
+    float2 X, Y, Z;
+    long long pix[2];  // (a map may hold more than 2^31)
+    float d[2];
+};
+__device__ __forceinline__ Seen see_pair(const FrameP& F, const float* depth, int ax, int ay, int az) {
     const CamF& c = F.cam;
-    float bx = F.fb[0], by = F.fb[1], bz = F.fb[2];
-    float vx = ((float)ax + bx) * F.vox, vy = ((float)ay + by) * F.vox, vz = ((float)az + bz) * F.vox;
-    float X = F.R[0] * vx + F.R[1] * vy + F.R[2] * vz;
-    float Y = F.R[3] * vx + F.R[4] * vy + F.R[5] * vz;
-    float Z = F.R[6] * vx + F.R[7] * vy + F.R[8] * vz;
+    Seen o;
+    const float2 vx = mul2(add2(make_float2((float)ax, (float)(ax + 1)), dup2(F.fb[0])), dup2(F.vox));
+    const float vy = __fmul_rn(__fadd_rn((float)ay, F.fb[1]), F.vox), vz = __fmul_rn(__fadd_rn((float)az, F.fb[2]), F.vox);
+    o.X = fma2(dup2(F.R[2]), dup2(vz), fma2(dup2(F.R[0]), vx, dup2(__fmul_rn(F.R[1], vy))));
+    o.Y = fma2(dup2(F.R[5]), dup2(vz), fma2(dup2(F.R[3]), vx, dup2(__fmul_rn(F.R[4], vy))));
+    o.Z = fma2(dup2(F.R[8]), dup2(vz), fma2(dup2(F.R[6]), vx, dup2(__fmul_rn(F.R[7], vy))));
     // projection (unified model + distortion) and nearest pixel
-    float n = sqrtf(fmaf(X, X, fmaf(Y, Y, Z * Z)));
-    float inv = 1.0f / fmaf(c.xi, n, Z);
-    float mx = X * inv, my = Y * inv;
-    float r2 = fmaf(mx, mx, my * my);
-    float rad = fmaf(r2, fmaf(c.k2, r2, c.k1), 1.0f);
-    float mxy = mx * my;
-    float xd = fmaf(mx, rad, fmaf(2.0f * c.p1, mxy, c.p2 * fmaf(2.0f * mx, mx, r2)));
-    float yd = fmaf(my, rad, fmaf(c.p1, fmaf(2.0f * my, my, r2), 2.0f * c.p2 * mxy));
-    float u = fmaf(c.fx, xd, c.cx), v = fmaf(c.fy, yd, c.cy);
-    if (!((Z > c.lim * n) && (r2 <= c.r2_max))) return false;
-    float pu = floorf(u + 0.5f), pv = floorf(v + 0.5f);
-    if (!(pu >= 0.f && pv >= 0.f && pu < (float)c.width && pv < (float)c.height)) return false;
-    const size_t pix = (size_t)pv * c.width + (size_t)pu;
-    if (!PS_DCHECK(pix < (size_t)c.width * c.height, CHK_PIXEL)) return false;
-    float d = __ldg(&depth[pix]);
-    if (!(d > 0.f) || !(d < 3.0e38f)) return false;
-    // |X_d| in voxel units: (a + b)^2 = a^2 (exact int) + (2a + b) b
-    int A2 = ax * ax + ay * ay + az * az;
-    float Bs = fmaf(fmaf(2.0f, (float)ax, bx), bx, fmaf(fmaf(2.0f, (float)ay, by), by, fmaf(2.0f, (float)az, bz) * bz));
-    float y = sqrtf((float)A2 + Bs);
-    float p = y * y;
-    float pe = fmaf(y, y, -p);  // p + pe = y^2 exactly
-    float diff = A2 < (1 << 24) ? (float)A2 - p : (float)(A2 - __float2int_rn(p));
-    float corr = ((diff - pe) + Bs) / (2.0f * y);  // |X_d| = y + corr (voxel units)
-    // eta = d - vox * (y + corr), with the product vox * y split exactly
-    float q = F.vox * y;
-    float qe = fmaf(F.vox, y, -q);
-    *eta_out = ((d - q) - qe) - fmaf(F.vox_lo, y, F.vox * corr);
-    *pix_out = pix;
-    Xc[0] = X;
-    Xc[1] = Y;
-    Xc[2] = Z;
-    return true;
-}
-
-// eta of a voxel at integer offset (ax, ay, az) from the camera voxel whose
-// pixel's depth is d (observe_voxel's arithmetic).
-__device__ __forceinline__ float voxel_eta(const FrameP& F, int ax, int ay, int az, float d) {
-    const float bx = F.fb[0], by = F.fb[1], bz = F.fb[2];
-    int A2 = ax * ax + ay * ay + az * az;
-    float Bs = fmaf(fmaf(2.0f, (float)ax, bx), bx, fmaf(fmaf(2.0f, (float)ay, by), by, fmaf(2.0f, (float)az, bz) * bz));
-    float y = sqrt_rn((float)A2 + Bs);
-    float p = y * y;
-    float pe = fmaf(y, y, -p);  // p + pe = y^2 exactly
-    float diff = A2 < (1 << 24) ? (float)A2 - p : (float)(A2 - __float2int_rn(p));
-    const float y2 = 2.0f * y;
-    float corr = div_rn((diff - pe) + Bs, y2, rcp_rn(y2));  // |X_d| = y + corr (voxel units)
-    float q = F.vox * y;
-    float qe = fmaf(F.vox, y, -q);
-    return ((d - q) - qe) - fmaf(F.vox_lo, y, F.vox * corr);
-}
-
-// Eq. 2 on two voxels, (ax, ay, az) and its +x neighbour: observe_voxel's
-// operations, the projection on packed pairs with branch-free quotients and
-// roots (the general forms' slow paths made the voxels of a thread wait for
-// each other: ring-type maps of 2 cm voxels were bound by that, not by HBM).
-__device__ __forceinline__ void update_pair(const FrameP& F, const float* depth, int ax, int ay, int az, float4& pr) {
-    const CamF& c = F.cam;
-    const float2 vx = make_float2(((float)ax + F.fb[0]) * F.vox, ((float)(ax + 1) + F.fb[0]) * F.vox);
-    const float vy = ((float)ay + F.fb[1]) * F.vox, vz = ((float)az + F.fb[2]) * F.vox;
-    const float2 X = fma2(dup2(F.R[2]), dup2(vz), fma2(dup2(F.R[0]), vx, dup2(F.R[1] * vy)));
-    const float2 Y = fma2(dup2(F.R[5]), dup2(vz), fma2(dup2(F.R[3]), vx, dup2(F.R[4] * vy)));
-    const float2 Z = fma2(dup2(F.R[8]), dup2(vz), fma2(dup2(F.R[6]), vx, dup2(F.R[7] * vy)));
-    const float2 n = sqrt_rn2(fma2(X, X, fma2(Y, Y, mul2(Z, Z))));
-    const float2 inv = rcp_rn2(fma2(dup2(c.xi), n, Z));
-    const float2 mx = mul2(X, inv), my = mul2(Y, inv);
+    const float2 n = sqrt_rn2(fma2(o.X, o.X, fma2(o.Y, o.Y, mul2(o.Z, o.Z))));
+    const float2 inv = rcp_rn2(fma2(dup2(c.xi), n, o.Z));
+    const float2 mx = mul2(o.X, inv), my = mul2(o.Y, inv);
     const float2 r2 = fma2(mx, mx, mul2(my, my));
     const float2 rad = fma2(r2, fma2(dup2(c.k2), r2, dup2(c.k1)), dup2(1.0f));
     const float2 mxy = mul2(mx, my);
@@ -366,20 +314,50 @@ __device__ __forceinline__ void update_pair(const FrameP& F, const float* depth,
     const float2 ln = mul2(dup2(c.lim), n);
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-        const float pu = floorf((q ? u.y : u.x) + 0.5f), pv = floorf((q ? v.y : v.x) + 0.5f);
-        const bool ok = (q ? Z.y > ln.y : Z.x > ln.x) && (q ? r2.y : r2.x) <= c.r2_max && pu >= 0.f && pv >= 0.f &&
-                        pu < (float)c.width && pv < (float)c.height;
-        const long long pix = ok ? (long long)(int)pv * c.width + (int)pu : 0;  // a map may hold more than 2^31
-        if (!PS_DCHECK(pix >= 0 && pix < (long long)c.width * c.height, CHK_PIXEL)) continue;
-        const float d = ok ? __ldg(&depth[pix]) : 0.f;
-        if (!(d > 0.f) || !(d < 3.0e38f)) continue;
-        const float eta = voxel_eta(F, ax + q, ay, az, d);
+        const float pu = floorf(__fadd_rn(q ? u.y : u.x, 0.5f)), pv = floorf(__fadd_rn(q ? v.y : v.x, 0.5f));
+        bool ok = (q ? o.Z.y > ln.y : o.Z.x > ln.x) && (q ? r2.y : r2.x) <= c.r2_max && pu >= 0.f && pv >= 0.f &&
+                  pu < (float)c.width && pv < (float)c.height;
+        o.pix[q] = ok ? (long long)(int)pv * c.width + (int)pu : 0;
+        ok = PS_DCHECK(o.pix[q] >= 0 && o.pix[q] < (long long)c.width * c.height, CHK_PIXEL) && ok;
+        const float d = ok ? __ldg(&depth[o.pix[q]]) : 0.f;
+        o.d[q] = d > 0.f && d < 3.0e38f ? d : 0.f;
+    }
+    return o;
+}
+
+// eta of a voxel at integer offset (ax, ay, az) from the camera voxel whose
+// pixel's depth is d; eta < -mu is left to the caller.
+__device__ __forceinline__ float voxel_eta(const FrameP& F, int ax, int ay, int az, float d) {
+    const float bx = F.fb[0], by = F.fb[1], bz = F.fb[2];
+    // |X_d| in voxel units: (a + b)^2 = a^2 (exact int) + (2a + b) b
+    const int A2 = ax * ax + ay * ay + az * az;
+    const float Bs = __fmaf_rn(__fmaf_rn(2.0f, (float)ax, bx), bx,
+                               __fmaf_rn(__fmaf_rn(2.0f, (float)ay, by), by, __fmul_rn(__fmaf_rn(2.0f, (float)az, bz), bz)));
+    const float y = sqrt_rn(__fadd_rn((float)A2, Bs));
+    const float p = __fmul_rn(y, y);
+    const float pe = __fmaf_rn(y, y, -p);  // p + pe = y^2 exactly
+    const float diff = A2 < (1 << 24) ? __fsub_rn((float)A2, p) : (float)(A2 - __float2int_rn(p));
+    const float y2 = __fmul_rn(2.0f, y);
+    const float corr = div_rn(__fadd_rn(__fsub_rn(diff, pe), Bs), y2, rcp_rn(y2));  // |X_d| = y + corr (voxel units)
+    // eta = d - vox * (y + corr), with the product vox * y split exactly
+    const float q = __fmul_rn(F.vox, y);
+    const float qe = __fmaf_rn(F.vox, y, -q);
+    return __fsub_rn(__fsub_rn(__fsub_rn(d, q), qe), __fmaf_rn(F.vox_lo, y, __fmul_rn(F.vox, corr)));
+}
+
+// Eq. 2 on two voxels, (ax, ay, az) and its +x neighbour.
+__device__ __forceinline__ void update_pair(const FrameP& F, const float* depth, int ax, int ay, int az, float4& pr) {
+    const Seen o = see_pair(F, depth, ax, ay, az);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        if (!(o.d[q] > 0.f)) continue;
+        const float eta = voxel_eta(F, ax + q, ay, az, o.d[q]);
         if (eta < -F.mu) continue;
-        const float sdf = fminf(1.0f, eta * F.inv_mu);
+        const float sdf = fminf(1.0f, __fmul_rn(eta, F.inv_mu));
         float& D = q ? pr.z : pr.x;
         float& w = q ? pr.w : pr.y;
         const float w1 = w + 1.0f;
-        D = div_rn(fmaf(w, D, sdf), w1, rcp_rn(w1));
+        D = div_rn(__fmaf_rn(w, D, sdf), w1, rcp_rn(w1));
         w = fminf(w1, F.w_max);
     }
 }
@@ -1120,15 +1098,18 @@ __global__ void __launch_bounds__(256) dense_fuse_bwd_kernel(const __grid_consta
                   gz = (int)(b / ((long long)nbx * nby)) * B + (v >> 6);
         const float g = PAIRS ? reinterpret_cast<const float2*>(gD)[i].x : gD[i];
         float out = g;
-        float eta, Xc[3];
-        size_t pix;
-        if (observe_voxel(F, depth, gx - F.ic[0], gy - F.ic[1], gz - F.ic[2], &eta, &pix, Xc) && !(eta < -F.mu)) {
+        const int ax = gx - F.ic[0], ay = gy - F.ic[1], az = gz - F.ic[2];
+        const Seen o = see_pair(F, depth, ax, ay, az);  // (the first of the two is used)
+        const float eta = voxel_eta(F, ax, ay, az, o.d[0]);
+        if (o.d[0] > 0.f && !(eta < -F.mu)) {
+            const float Xc[3] = {o.X.x, o.Y.x, o.Z.x};
             const float w = vox_in[i].y;
             out = g * w / (w + 1.0f);
             if (eta < F.mu && g != 0.f) {
                 const float ge = g / (F.mu * (w + 1.0f));
-                if (g_depth) atomicAdd(&g_depth[pix], ge);
-                const float s = -ge / sqrtf(Xc[0] * Xc[0] + Xc[1] * Xc[1] + Xc[2] * Xc[2]);
+                if (g_depth) atomicAdd(&g_depth[o.pix[0]], ge);
+                // (roundings written out: contracted otherwise, the sums that cancel in the pose's rotation part move)
+                const float s = -ge / sqrtf(__fadd_rn(__fmaf_rn(Xc[0], Xc[0], __fmul_rn(Xc[1], Xc[1])), __fmul_rn(Xc[2], Xc[2])));
                 const float gx3[3] = {s * Xc[0], s * Xc[1], s * Xc[2]};
                 acc[0] += Xc[1] * gx3[2] - Xc[2] * gx3[1];
                 acc[1] += Xc[2] * gx3[0] - Xc[0] * gx3[2];
