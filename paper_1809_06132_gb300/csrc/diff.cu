@@ -247,6 +247,23 @@ __device__ __forceinline__ void pair_windows(const float* R, const float2* W, in
         }
 }
 
+// ZNCC of both planes from the window sums, and the root of the variances'
+// product that divides it.  Variances whose product overflows have an infinite
+// root, and no correlation.
+struct Corr {
+    float2 z, s;
+};
+__device__ __forceinline__ Corr correlation(float va, float2 vb, float2 cov) {
+    const float inf = __int_as_float(0x7f800000);
+    const float2 p = mul2(dup2(va), vb);
+    Corr o;
+    o.s = sqrt_rn2(p);
+    o.z = div_rn2(cov, o.s, rcp_rn2(o.s));
+    if (p.x == inf) o.s.x = inf, o.z.x = __fmul_rn(cov.x, 0.f);
+    if (p.y == inf) o.s.y = inf, o.z.y = __fmul_rn(cov.y, 0.f);
+    return o;
+}
+
 // The tile's reference samples (zero outside the image).
 template <class G>
 __device__ __forceinline__ void load_ref(const DiffP& P, int x0, int y0, float* R) {
@@ -327,7 +344,7 @@ __global__ void __launch_bounds__(FG * ST, 1) soft_fwd_kernel(const __grid_const
                 for (int i = 0; i < PX; ++i) {
                     const bool ok0 = !isnan(mb[i].x) && !(va[i] < lim || vb[i].x < lim);
                     const bool ok1 = !isnan(mb[i].y) && !(va[i] < lim || vb[i].y < lim);
-                    const float2 s = sqrt_rn2(mul2(dup2(va[i]), vb[i])), z = div_rn2(cov[i], s, rcp_rn2(s));
+                    const float2 z = correlation(va[i], vb[i], cov[i]).z;
                     const float c0 = 0.5f * (1.0f - z.x), c1 = 0.5f * (1.0f - z.y);
                     if (ok0 && c0 < best[i].x) best[i].x = c0;
                     if (ok1 && c1 < best[i].y) best[i].y = c1;
@@ -573,8 +590,9 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
             float2 ss[PX], zz[PX];
 #pragma unroll
             for (int i = 0; i < PX; ++i) {
-                ss[i] = sqrt_rn2(mul2(dup2(va[i]), v2[i]));
-                zz[i] = div_rn2(c2[i], ss[i], rcp_rn2(ss[i]));
+                const Corr o = correlation(va[i], v2[i], c2[i]);
+                ss[i] = o.s;
+                zz[i] = o.z;
             }
 #pragma unroll
             for (int i = 0; i < PX; ++i)
@@ -610,9 +628,10 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
                 const float gC = gE[i] * div_rn(-s * (rho_k - E[i]), P.T, inv_T) + gs[i] * s;
                 const float gz = -0.5f * gC, gzz = gz * z[i][q];
                 const bool on = jb[i][q] >= 0;
-                ka[q] = on ? div_rn(gz, sab[i][q], rcp_rn(sab[i][q])) : 0.f;
-                kza[q] = on ? div_rn(gzz, va[i], rcp_rn(va[i])) : 0.f;
-                kzb[q] = on ? div_rn(gzz, vb[i][q], rcp_rn(vb[i][q])) : 0.f;
+                const bool finite = on && sab[i][q] < inf;  // (otherwise all three are zero)
+                ka[q] = finite ? div_rn(gz, sab[i][q], rcp_rn(sab[i][q])) : 0.f;
+                kza[q] = finite ? div_rn(gzz, va[i], rcp_rn(va[i])) : 0.f;
+                kzb[q] = finite ? div_rn(gzz, vb[i][q], rcp_rn(vb[i][q])) : 0.f;
                 mac[q] = on ? ma[i] - ca : 0.f;
                 mbc[q] = on ? mb[i][q] - (q ? cb.y : cb.x) : 0.f;
             }

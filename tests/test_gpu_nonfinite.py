@@ -54,3 +54,21 @@ def test_a_range_beyond_the_largest_block_count():
     m, depth, pose = _far_map(None)
     m.integrate(depth, pose)
     assert m.status() == P.PS_ERR_CAPACITY and m.count() == 0    # no local map: no key holds such a block
+
+
+def test_variances_whose_product_overflows():
+    # a correlation over an infinite deviation is 0: every such plane costs 1/2
+    T = 0.05
+    wl = scenes.diff(5, width=64, height=48, n_planes=6)
+    imgs, _ = scenes.FrameSource(wl).frame(0)
+    dev = [i.float().cuda() / 255.0 for i in imgs]
+    sw = P.SoftSweep(wl.rig, wl.levels[0], temperature=T)
+    usual, _, _ = sw.forward(dev)
+    big = [1e12 * d for d in dev]
+    r, c, aux = sw.forward(big)
+    gi, gp = sw.backward(big, None, aux, torch.ones_like(r), torch.ones_like(c))
+    assert (r > 0)[usual > 0].all() and torch.isfinite(r).all() and torch.isfinite(c).all()
+    # the soft minimum of n equal costs is 1/2 - T log n: exp((1/2 - c) / T) is n, to the rounding of c over T
+    n = torch.exp((0.5 - c[usual > 0]) / T)
+    assert ((n - n.round()).abs() <= n * 2.0 ** -22 / T).all() and (n.round() >= 1).all() and (n.round() <= 6).all()
+    assert all((g == 0).all() for g in gi) and (gp == 0).all()
