@@ -38,6 +38,7 @@
 // softmax, box sums and the pose accumulators keep one order whatever the
 // tiling.
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 #include <cstring>
 #include <type_traits>
@@ -814,7 +815,7 @@ int fill_params(const psdiff_t* h, const float* const* images, const ps_pose* re
     P.rho = h->rho;
     P.K = h->K;
     P.n_cams = h->n_cams;
-    P.T = (float)h->T;
+    P.T = std::max((float)h->T, FLT_MIN);  // (1 / T of a subnormal one overflows; both leave one plane's weight alone)
     P.rays = h->rays;
     P.planes = h->planes;
     PS_ARG(images != nullptr && images[0] != nullptr, "psdiff: images[0] is NULL");

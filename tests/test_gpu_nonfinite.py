@@ -72,3 +72,13 @@ def test_variances_whose_product_overflows():
     n = torch.exp((0.5 - c[usual > 0]) / T)
     assert ((n - n.round()).abs() <= n * 2.0 ** -22 / T).all() and (n.round() >= 1).all() and (n.round() <= 6).all()
     assert all((g == 0).all() for g in gi) and (gp == 0).all()
+
+
+@pytest.mark.parametrize("T", [1e-39, 1e-42])
+def test_a_temperature_below_the_smallest_normal_number(T):
+    # costs differ by 2^-25 or more: any such temperature takes the plane of the lowest cost alone
+    wl = scenes.diff(5, width=48, height=40, n_planes=6)
+    imgs, _ = scenes.FrameSource(wl).frame(0)
+    dev = [i.float().cuda() / 255.0 for i in imgs]
+    a, b = (P.SoftSweep(wl.rig, wl.levels[0], temperature=t).forward(dev) for t in (T, 1e-30))
+    assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1]) and (a[0] > 0).any()
