@@ -561,7 +561,8 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
 #pragma unroll
     for (int i = 0; i < RPT; ++i) gR[i] = 0.f;
     const int qc = (RHO + TH / 2) * HWC + RHO + SW / 2;  // centre of the tile
-    const float ca = R[(RHO + TH / 2) * G::RS + RHO + SW / 2];
+    auto finite = [&](float v) { return fabsf(v) < inf ? v : 0.f; };  // a centre that is none must not reach all of the tile
+    const float ca = finite(R[(RHO + TH / 2) * G::RS + RHO + SW / 2]);
     for (int k = 0; k < P.K; k += 2) {
         const int np = min(2, P.K - k);
         const PlaneD pl0 = P.planes[k], pl1 = P.planes[k + np - 1];
@@ -571,7 +572,7 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
         // the per-camera centre of this pair's warped samples (a broadcast read)
         auto centre = [&](int j) {
             const float2 c = W2[j * NPOS + qc];
-            return make_float2(isnan(c.x) ? 0.f : c.x, isnan(c.y) ? 0.f : c.y);
+            return make_float2(finite(c.x), finite(c.y));
         };
         // 2. cost, camera and coefficients
         float best[PX][2], z[PX][2], mb[PX][2], vb[PX][2], sab[PX][2];
@@ -745,7 +746,8 @@ __global__ void __launch_bounds__(ST, 2) soft_bwd_kernel(const __grid_constant__
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
             const int p = tid + i * ST, x = x0 + p % HWC, y = y0 + p / HWC;
-            if (p < NPOS && gR[i] != 0.f && PS_DCHECK(x >= 0 && y >= 0 && x < P.W && y < P.H, CHK_PIXEL))
+            // (outside the image gR is zero, or no number where an intensity is infinite)
+            if (p < NPOS && gR[i] != 0.f && x >= 0 && y >= 0 && x < P.W && y < P.H)
                 atomicAdd(&g_ref[(size_t)y * P.W + x], gR[i]);
         }
     }

@@ -82,3 +82,31 @@ def test_a_temperature_below_the_smallest_normal_number(T):
     dev = [i.float().cuda() / 255.0 for i in imgs]
     a, b = (P.SoftSweep(wl.rig, wl.levels[0], temperature=t).forward(dev) for t in (T, 1e-30))
     assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1]) and (a[0] > 0).any()
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), float("-inf")])
+@pytest.mark.parametrize("window,x,y", [(5, 8, 8), (9, 24, 24), (7, 24, 8)])
+def test_a_tile_centre_that_is_no_number(window, x, y, value):
+    # the pixel that a tile's intensities are taken relative to, in tiles whose halo leaves the image:
+    # nothing is written outside the image's gradient, and inside only its own value is none
+    w = h = 32
+    wl = scenes.diff(3, width=w, height=h, n_planes=6)
+    lv = dataclasses.replace(wl.levels[0], window=window)
+    imgs, _ = scenes.FrameSource(wl).frame(0)
+    dev = [i.float().cuda() / 255.0 for i in imgs]
+    dev[0][y, x] = value
+    sw = P.SoftSweep(wl.rig, lv)
+    r, c, aux = sw.forward(dev)
+    one = torch.ones_like(r)
+    pad = 16 * w
+    buf = torch.zeros(2 * pad + h * w, device="cuda")
+    g = [buf[pad:pad + h * w]] + [torch.zeros_like(d) for d in dev[1:]]
+    gp = torch.zeros((2, 6), dtype=torch.float64, device="cuda")
+    ims, poses = sw._args(dev, None)
+    ptrs = (type(ims))(*[t.data_ptr() for t in g])
+    assert P.load().psdiff_backward(sw.h, ims, poses, aux.data_ptr(), one.data_ptr(), one.data_ptr(), ptrs, gp.data_ptr(),
+                                    torch.cuda.current_stream().cuda_stream) == P.PS_OK
+    assert (buf[:pad] == 0).all() and (buf[pad + h * w:] == 0).all()
+    bad = ~torch.isfinite(g[0].view(h, w))
+    bad[y, x] = False
+    assert not bad.any() and (g[0].nan_to_num(0, 0, 0) != 0).any()
