@@ -364,7 +364,9 @@ __device__ __forceinline__ void update_pair(const FrameP& F, const float* depth,
 
 // 32 registers (8 CTAs, the whole register file, per SM): at 2 cm voxels (40 k
 // listed blocks, 330 MB read and written) 98 us a frame against 107 with 6
-// CTAs and 130 with the general divisions and roots.
+// CTAs and 130 with the general divisions and roots.  That is about half of
+// the copy bandwidth: issue is active 66 % of the time and the XU pipe 22 %,
+// so instructions per voxel and the chain list -> key -> voxels bound it.
 __global__ void __launch_bounds__(IT, 8) integrate_kernel(const __grid_constant__ FrameP F, TsdfDev T,
                                                        const float* depth) {
     int nv = *T.n_vis;
