@@ -253,6 +253,8 @@ def _dense(t: torch.Tensor, stream) -> torch.Tensor:
     """t, or a contiguous copy of it made on the stream of the call that reads it."""
     if t.is_contiguous() or stream is None:
         return t.contiguous()
+    if not isinstance(stream, torch.cuda.Stream):   # any object with a cuda_stream is taken
+        stream = torch.cuda.ExternalStream(stream.cuda_stream, device=t.device)
     with torch.cuda.stream(stream):
         return t.contiguous()
 

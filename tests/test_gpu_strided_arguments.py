@@ -65,3 +65,24 @@ def test_strided_blocks_of_a_map():
     k, D, W = m.extract()
     order = torch.argsort(k[:, 0])
     assert torch.equal(k[order], keys) and torch.equal(D[order], dw[..., 0]) and torch.equal(W[order], dw[..., 1])
+
+
+@pytest.mark.parametrize("foreign", [False, True])
+def test_strided_gradients_on_another_stream(foreign):
+    wl = scenes.diff(1, width=64, height=48, n_planes=8)
+    imgs, _ = scenes.FrameSource(wl).frame(0)
+    dev = [i.float().cuda() / 255.0 for i in imgs]
+    sw = P.SoftSweep(wl.rig, wl.levels[0])
+    r, c, aux = sw.forward(dev)
+    g = torch.randn((64, 48), device="cuda")
+    expect, _ = sw.backward(dev, None, aux, g.t().contiguous(), (2 * g).t().contiguous())
+    side = torch.cuda.Stream()
+
+    class Handle:           # what another library's stream looks like
+        cuda_stream = side.cuda_stream
+    for _ in range(3):
+        torch.cuda.synchronize()
+        got, _ = sw.backward(dev, None, aux, g.t(), (2 * g).t(), stream=Handle() if foreign else side)
+        torch.cuda.synchronize()
+        for a, b in zip(got, expect):
+            assert (a - b).norm() <= 1e-5 * b.norm() and b.any()
