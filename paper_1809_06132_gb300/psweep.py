@@ -9,6 +9,7 @@ There is no fallback: if the library cannot be loaded, importing it fails.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes as C
 import os
 from typing import Optional, Sequence
@@ -249,14 +250,23 @@ def _dev(t: torch.Tensor, dtype, name: str) -> int:
     return t.data_ptr()
 
 
-def _dense(t: torch.Tensor, stream) -> torch.Tensor:
-    """t, or a contiguous copy of it made on the stream of the call that reads it."""
-    if t.is_contiguous() or stream is None:
-        return t.contiguous()
+def _on(stream, device):
+    """Context in which the buffers and copies that a call on `stream` needs are
+    made: cleared or filled on another stream they would race with its kernels."""
+    if stream is None:
+        return contextlib.nullcontext()
     if not isinstance(stream, torch.cuda.Stream):   # any object with a cuda_stream is taken
-        stream = torch.cuda.ExternalStream(stream.cuda_stream, device=t.device)
-    with torch.cuda.stream(stream):
-        return t.contiguous()
+        stream = torch.cuda.ExternalStream(stream.cuda_stream, device=device)
+    return torch.cuda.stream(stream)
+
+
+def _returned(stream, *tensors):
+    """Results made on `stream` go to the caller's current one: their memory is
+    not used again before what it then does with them is done."""
+    if stream is not None:
+        for t in tensors:
+            if t is not None:
+                t.record_stream(torch.cuda.current_stream(t.device))
 
 
 def level_shape(ref, lv):
@@ -656,7 +666,8 @@ class Tsdf:
     def load_blocks(self, keys: torch.Tensor, D: torch.Tensor, W: torch.Tensor, stream=None):
         """Insert or overwrite blocks (checkpoint resume, swap-in)."""
         n = keys.shape[0]
-        keys, D, W = (_dense(t, stream) for t in (keys, D, W))
+        with _on(stream, keys.device):
+            keys, D, W = keys.contiguous(), D.contiguous(), W.contiguous()
         _check(load().tsdf_load(self.h, _dev(keys, torch.int32, "keys"), _dev(D, torch.float32, "D"),
                                 _dev(W, torch.float32, "W"), n, _stream_ptr(stream)))
 
@@ -807,18 +818,20 @@ class SoftSweep:
     def backward(self, images, poses, aux, g_range=None, g_cost=None, stream=None):
         """(per-image gradients, (n_cams, 6) float64 pose gradients (w, v))."""
         ims, ps = self._args(images, poses)
-        # a tensor of its own per image (slices of one would share its memory and
-        # version, and refuse some in-place operations), cleared in one launch
-        gi = [torch.empty_like(im) for im in images]
-        torch._foreach_zero_(gi)
+        with _on(stream, images[0].device):
+            # a tensor of its own per image (slices of one would share its memory and
+            # version, and refuse some in-place operations), cleared in one launch
+            gi = [torch.empty_like(im) for im in images]
+            torch._foreach_zero_(gi)
+            gp = torch.zeros((len(self.rig.cams), 6), dtype=torch.float64, device=images[0].device)
+            g_range = g_range.contiguous() if g_range is not None else None
+            g_cost = g_cost.contiguous() if g_cost is not None else None
         gptr = (C.c_void_p * len(gi))(*[g.data_ptr() for g in gi])
-        gp = torch.zeros((len(self.rig.cams), 6), dtype=torch.float64, device=images[0].device)
-        g_range = _dense(g_range, stream) if g_range is not None else None
-        g_cost = _dense(g_cost, stream) if g_cost is not None else None
         gr = _dev(g_range, torch.float32, "g_range") if g_range is not None else None
         gc = _dev(g_cost, torch.float32, "g_cost") if g_cost is not None else None
         _check(load().psdiff_backward(self.h, ims, ps, _dev(aux, torch.float32, "aux"), gr, gc, gptr,
                                       gp.data_ptr(), _stream_ptr(stream)))
+        _returned(stream, *gi, gp)
         return gi, gp
 
 
@@ -855,11 +868,12 @@ def soft_depth(sweep: SoftSweep, images, delta: Optional[torch.Tensor] = None, b
 def tsdf_dense_fuse_backward(voxels_in, dims, origin, voxel_size, mu, w_max, depth, cam, world_to_cam, g_D_out,
                              want_depth: bool = True, want_pose: bool = True, stream=None):
     """(dL/dD_in per voxel, dL/ddepth, (6,) float64 pose gradient) of one fusion step."""
-    g_D_out = _dense(g_D_out, stream)
+    with _on(stream, voxels_in.device):
+        g_D_out = g_D_out.contiguous()
+        gin = torch.empty(g_D_out.shape, dtype=torch.float32, device=voxels_in.device)
+        gd = torch.zeros(depth.shape, dtype=torch.float32, device=depth.device) if want_depth else None
+        gp = torch.zeros(6, dtype=torch.float64, device=depth.device) if want_pose else None
     gD = _dev(g_D_out, torch.float32, "g_D_out")
-    gin = torch.empty(g_D_out.shape, dtype=torch.float32, device=voxels_in.device)
-    gd = torch.zeros(depth.shape, dtype=torch.float32, device=depth.device) if want_depth else None
-    gp = torch.zeros(6, dtype=torch.float64, device=depth.device) if want_pose else None
     dims_a = (C.c_int32 * 3)(*[int(v) for v in dims])
     org = (C.c_double * 3)(*[float(v) for v in origin])
     _check(load().tsdf_dense_fuse_backward(_dev(voxels_in, torch.float32, "voxels_in"), dims_a, org,
@@ -868,6 +882,7 @@ def tsdf_dense_fuse_backward(voxels_in, dims, origin, voxel_size, mu, w_max, dep
                                            C.byref(pose(world_to_cam)), gD, gin.data_ptr(),
                                            gd.data_ptr() if gd is not None else None,
                                            gp.data_ptr() if gp is not None else None, _stream_ptr(stream)))
+    _returned(stream, gin, gd, gp)
     return gin, gd, gp
 
 

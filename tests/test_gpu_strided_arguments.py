@@ -86,3 +86,28 @@ def test_strided_gradients_on_another_stream(foreign):
         torch.cuda.synchronize()
         for a, b in zip(got, expect):
             assert (a - b).norm() <= 1e-5 * b.norm() and b.any()
+
+
+def test_gradients_are_cleared_on_the_stream_of_the_call():
+    # the current stream is busy: what is cleared there is cleared after the kernel has added to it
+    wl = scenes.diff(1, width=64, height=48, n_planes=8)
+    imgs, _ = scenes.FrameSource(wl).frame(0)
+    dev = [i.float().cuda() / 255.0 for i in imgs]
+    sw = P.SoftSweep(wl.rig, wl.levels[0])
+    r, c, aux = sw.forward(dev)
+    one = torch.ones_like(r)
+    ei, ep = sw.backward(dev, None, aux, one, one)
+    cam = scenes.Camera(xi=1.0, fx=40.0, fy=40.0, cx=24.0, cy=20.0, width=48, height=40)
+    p = TsdfParams(voxel_size=0.1, mu=0.3, w_max=4.0, dense_dim=(16, 16, 16), origin=(-0.8, -0.8, 1.2))
+    args = (torch.rand((8, 512, 2), device="cuda"), p.dense_dim, p.origin, p.voxel_size, p.mu, p.w_max,
+            2.0 + 0.1 * torch.rand((40, 48), device="cuda"), cam, Pose(rot_xyz(0.01, 0.02, 0.0), np.array([0.02, -0.01, 0.03])),
+            torch.randn((8, 512), device="cuda"))
+    expect = ei + [ep] + list(tsdf_dense_fuse_backward(*args))
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    torch.cuda._sleep(200_000_000)          # about 0.1 s
+    gi, gp = sw.backward(dev, None, aux, one, one, stream=side)
+    got = gi + [gp] + list(tsdf_dense_fuse_backward(*args, stream=side))
+    torch.cuda.synchronize()
+    for a, b in zip(got, expect):
+        assert (a - b).norm() <= 1e-5 * b.norm() and b.any()
